@@ -13,7 +13,7 @@
 //   4. Per tile row, in chunks of rows: the rows expanded into per-tile instance lists in
 //      depth order, and the per-tile [start, end) ranges.
 //
-// The radix sort is reduce-then-scan (upsweep histogram, one-CTA scan, downsweep
+// The radix sort is reduce-then-scan (upsweep histogram, one scan CTA per digit, downsweep
 // scatter) with persistent CTAs that own contiguous tile ranges: no CTA ever waits on
 // another.  The upsweep counts runs of equal digits per thread; ranking inside a tile is
 // stable (warp multi-split by digit-bit ballots + per-warp counters) and the scatter goes
@@ -26,6 +26,7 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortIPT = 8;
 constexpr int kSortTile = kSortThreads * kSortIPT;  // 2048 items
+constexpr int kSortNoScan = 16;  // CTAs up to which a pass needs no scan kernel
 
 __device__ __forceinline__ void cta_tiles(uint32_t count, uint32_t &lo, uint32_t &hi) {
   uint32_t ntiles = (count + kSortTile - 1) / kSortTile;
@@ -121,24 +122,6 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t *ws, ui
   return r;
 }
 
-// Exclusive scan of `n` entries in place with one CTA of 1024 threads; the total goes to
-// *d_total when non-null.
-__global__ void __launch_bounds__(1024) scan_single_cta(uint32_t *data, int n, uint32_t *d_total) {
-  __shared__ uint32_t ws[33];
-  const int seg = (n + 1023) / 1024;
-  const int b = threadIdx.x * seg, e = min(b + seg, n);
-  uint32_t s = 0;
-  for (int i = b; i < e; ++i) s += data[i];
-  uint32_t tot;
-  uint32_t run = block_excl_scan(s, ws, &tot);
-  for (int i = b; i < e; ++i) {
-    uint32_t v = data[i];
-    data[i] = run;
-    run += v;
-  }
-  if (d_total && threadIdx.x == 0) *d_total = tot;
-}
-
 // Values are 4-byte item ids, or (WIDE) the 8-byte payload of a support row.
 template <bool WIDE>
 struct SortVal {
@@ -174,7 +157,27 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_downsweep(SortPass p) {
 
   uint32_t lo, hi;
   cta_tiles(pass_count(p), lo, hi);
-  for (int d = threadIdx.x; d < R; d += kSortThreads) s_base[d] = p.hist[size_t(d) * p.G + blockIdx.x];
+  {  // first output of each digit: the lower digits' items, then the lower CTAs' of this digit
+    static_assert(R <= kSortThreads, "one digit per thread");
+    uint32_t before = 0, total = 0;
+    if (threadIdx.x < R) {
+      const uint32_t *row = p.hist + size_t(threadIdx.x) * p.G;
+      if (p.G > kSortNoScan) {
+        before = row[blockIdx.x];
+        total = p.hist[size_t(R) * p.G + threadIdx.x];
+      } else {
+        for (int c = 0; c < p.G; ++c) {
+          const uint32_t n = row[c];
+          total += n;
+          before += c < int(blockIdx.x) ? n : 0u;
+        }
+      }
+    }
+    uint32_t all;
+    const uint32_t lower = block_excl_scan(total, s_ws, &all);
+    if (threadIdx.x < R) s_base[threadIdx.x] = lower + before;
+    if (p.d_total && blockIdx.x == 0 && threadIdx.x == 0) *p.d_total = all;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
 
@@ -312,72 +315,47 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_downsweep(SortPass p) {
   }
 }
 
-// Exclusive scan of the digit-major histogram [R][G] in place, in three steps: per-block
-// sums (one block per 2048 entries), a scan of the block sums, and the block-local scans.
-constexpr int kHistBlock = 2048;
+// Exclusive scan of one digit's counts over the CTAs, in place, and the digit's total (one
+// CTA per digit); the downsweep scans the R digit totals itself.
+constexpr int kSortMaxGrid = 1024;
 
-__global__ void __launch_bounds__(256) hist_reduce_kernel(const uint32_t *hist, int n, uint32_t *bsum) {
+__global__ void __launch_bounds__(256) hist_scan_kernel(uint32_t *hist, int G, uint32_t *digit_total) {
   __shared__ uint32_t ws[33];
-  const int b0 = blockIdx.x * kHistBlock;
-  uint32_t s = 0;
-  for (int i = b0 + threadIdx.x; i < min(b0 + kHistBlock, n); i += blockDim.x) s += hist[i];
-  uint32_t tot;
-  block_excl_scan(s, ws, &tot);
-  if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(1024) hist_bsum_kernel(uint32_t *bsum, int nb, uint32_t *d_total) {
-  __shared__ uint32_t ws[33];
-  const int per = (nb + 1023) / 1024;
-  const int b = threadIdx.x * per, e = min(b + per, nb);
-  uint32_t s = 0;
-  for (int i = b; i < e; ++i) s += bsum[i];
-  uint32_t tot;
-  uint32_t run = block_excl_scan(s, ws, &tot);
-  for (int i = b; i < e; ++i) {
-    const uint32_t v = bsum[i];
-    bsum[i] = run;
-    run += v;
-  }
-  if (d_total && threadIdx.x == 0) *d_total = tot;
-}
-
-__global__ void __launch_bounds__(256) hist_offsets_kernel(uint32_t *hist, int n, const uint32_t *bsum) {
-  __shared__ uint32_t ws[33];
-  const int b0 = blockIdx.x * kHistBlock;
-  constexpr int PER = kHistBlock / 256;
+  constexpr int PER = kSortMaxGrid / 256;
+  uint32_t *row = hist + size_t(blockIdx.x) * G;
   uint32_t v[PER], s = 0;
 #pragma unroll
   for (int j = 0; j < PER; ++j) {
-    const int i = b0 + threadIdx.x * PER + j;
-    v[j] = i < n ? hist[i] : 0u;
+    const int i = threadIdx.x * PER + j;
+    v[j] = i < G ? row[i] : 0u;
     s += v[j];
   }
   uint32_t tot;
-  uint32_t run = bsum[blockIdx.x] + block_excl_scan(s, ws, &tot);
+  uint32_t run = block_excl_scan(s, ws, &tot);
 #pragma unroll
   for (int j = 0; j < PER; ++j) {
-    const int i = b0 + threadIdx.x * PER + j;
-    if (i < n) hist[i] = run;
+    const int i = threadIdx.x * PER + j;
+    if (i < G) row[i] = run;
     run += v[j];
   }
+  if (threadIdx.x == 0) digit_total[blockIdx.x] = tot;
 }
 
 // One LSD pass: 8-bit digits over item ids (the depth sort), 4 to 8 bits over support
-// rows (the tile-row sort).
+// rows (the tile-row sort).  The grid is at most one CTA per 2,048 items.  Up to
+// kSortNoScan CTAs (32,768 items) every downsweep CTA reads the counts of all of them
+// instead of a scan kernel's offsets: two launches instead of three; the 720p frame's
+// 500,000 pairs (245 CTAs) are past the point where that reading costs more than the launch.
 template <int BITS, bool WIDE>
 static void sort_pass(const SortPass &p, cudaStream_t st) {
-  const int n = (1 << BITS) * p.G;
-  const int nb = (n + kHistBlock - 1) / kHistBlock;
-  uint32_t *bsum = p.hist + n;  // scratch after the histogram (the layout reserves 512*G + G)
   sort_upsweep<BITS><<<p.G, kSortThreads, 0, st>>>(p);
-  hist_reduce_kernel<<<nb, 256, 0, st>>>(p.hist, n, bsum);
-  hist_bsum_kernel<<<1, 1024, 0, st>>>(bsum, nb, p.d_total);
-  hist_offsets_kernel<<<nb, 256, 0, st>>>(p.hist, n, bsum);
+  if (p.G > kSortNoScan) hist_scan_kernel<<<1 << BITS, 256, 0, st>>>(p.hist, p.G, p.hist + (size_t(p.G) << BITS));
   sort_downsweep<BITS, WIDE><<<p.G, kSortThreads, 0, st>>>(p);
 }
 
-cudaError_t launch_sort_pass(const SortPass &p, cudaStream_t st) {
+cudaError_t launch_sort_pass(SortPass p, cudaStream_t st) {
+  const uint32_t need = (p.count_max + uint32_t(kSortTile) - 1u) / uint32_t(kSortTile);  // CTAs with work
+  p.G = need < uint32_t(p.G) ? (need ? int(need) : 1) : p.G;
   if (!p.wide) {
     if (p.bits != 8) return cudaErrorInvalidValue;
     sort_pass<8, false>(p, st);

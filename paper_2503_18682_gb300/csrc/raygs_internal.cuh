@@ -181,7 +181,7 @@ struct SortPass {
   int shift;
   int bits;                 // digit width of this pass (8 for item ids, 4-8 for support rows)
   int filter;               // drop kCulled keys; value = item index
-  uint32_t *hist;           // [512][G]
+  uint32_t *hist;           // [digits][G], then the digit totals
   int G;
   uint32_t *d_total;        // receives the number of items kept (nullable)
   // wide mode (tile-row sort of the support rows): 8-byte values (sorted pair position,
@@ -335,7 +335,7 @@ struct ParamGradParams {
 void note_cuda_error(cudaError_t e);
 
 cudaError_t launch_preprocess(const PrepParams &P, int num_sms, cudaStream_t st);
-cudaError_t launch_sort_pass(const SortPass &p, cudaStream_t st);
+cudaError_t launch_sort_pass(SortPass p, cudaStream_t st);
 cudaError_t launch_scan(const ScanJob &J, int G, cudaStream_t st);
 cudaError_t launch_rows(const RowsParams &R, int G, cudaStream_t st);
 cudaError_t launch_trow_scan(unsigned long long *trow_inst, uint2 *trow_ranges, int trows, Counters *c, uint32_t cap,
