@@ -66,7 +66,7 @@ raygs_status raygs_plan_create(const raygs_camera *cams, int32_t n_views, int64_
   if (!cams || n_views < 1 || n_views > RAYGS_MAX_VIEWS) return RAYGS_ERR_INVALID_ARG;
   if (n_gaussians < 0 || n_gaussians >= (int64_t(1) << 31)) return RAYGS_ERR_INVALID_ARG;
   if (int64_t(n_views) * n_gaussians >= (int64_t(1) << 32) - 1) return RAYGS_ERR_INVALID_ARG;
-  if (max_instances < 0 || max_instances >= (int64_t(1) << 32) - 4 * kEmitTile) return RAYGS_ERR_INVALID_ARG;
+  if (max_instances < 0 || max_instances >= (int64_t(1) << 32) - 8192) return RAYGS_ERR_INVALID_ARG;
   raygs_config cfg;
   if (cfg_in) cfg = *cfg_in; else raygs_config_default(&cfg);
   if (!config_valid(cfg)) return RAYGS_ERR_INVALID_ARG;
@@ -77,8 +77,8 @@ raygs_status raygs_plan_create(const raygs_camera *cams, int32_t n_views, int64_
   p->cams.assign(cams, cams + n_views);
   p->dcams.resize(n_views);
   int64_t tb = 0, trows = 0, pb = 0;
-  int max_tx = 0;
-  if (!plan_views(cams, n_views, cfg, p->dcams.data(), tb, trows, pb, max_tx)) {
+  int max_tx = 0, max_rows = 0;
+  if (!plan_views(cams, n_views, cfg, p->dcams.data(), tb, trows, pb, max_tx, max_rows)) {
     delete p;
     return RAYGS_ERR_INVALID_ARG;
   }
@@ -92,11 +92,12 @@ raygs_status raygs_plan_create(const raygs_camera *cams, int32_t n_views, int64_
   w.tiles = tb;
   w.trows = trows;
   w.max_tiles_x = max_tx;
+  w.max_rows = max_rows;
   w.cap = max_instances;
   w.num_sms = sms;
   w.G = sort_grid(sms);
   w.cfg = cfg;
-  w.L = make_layout(n_views, n_gaussians, tb, trows, max_instances, w.G, max_tx, cfg.enable_backward != 0,
+  w.L = make_layout(n_views, n_gaussians, tb, trows, max_instances, w.G, max_tx, max_rows, cfg.enable_backward != 0,
                     cams[0].mip == RAYGS_MIP_EXACT);
   p->total_pixels = pb;
   *out = p;
@@ -300,8 +301,8 @@ raygs_status raygs_debug_render_counted(raygs_plan *plan, float *rgb, float *T_f
 
 /* Device pointers of internal buffers (valid after bin_sort):
  * which: 0 depth keys [V*N], 1 rects [V*N] (uint2), 2 records [V*N] (64 B),
- *        3 sorted pair ids [n_visible], 4 support rows sorted by tile row [n_rows_kept]
- *        (uint2: sorted pair position, first tile column | run length << 16),
+ *        3 sorted pair ids [n_visible], 4 support rows listed by tile row [n_rows] (uint2:
+ *        sorted pair position, first tile column | run length << 16),
  *        5 instance lists (sorted pair positions, tile by tile), 6 tile ranges [tiles] (uint2),
  *        7 support ellipses [V*N] (32 B), 8 raw counters, 9 per-tile stop positions of the
  *        last instrumented render [tiles] (kCulled: the list ran out first) */
@@ -313,7 +314,7 @@ void *raygs_debug_buffer(raygs_plan *plan, int which) {
     case 1: return w.base + w.L.rect;
     case 2: return w.base + w.L.rec;
     case 3: return w.base + w.L.s1v[w.s1_final];
-    case 4: return w.base + w.L.rv[w.s2_rows];
+    case 4: return w.base + w.L.rows;
     case 5: return w.base + w.L.inst;
     case 6: return w.base + w.L.ranges;
     case 7: return w.base + w.L.ell;

@@ -57,8 +57,8 @@ extern "C" raygs_status raygs_render_noalloc(const raygs_camera *cams, int32_t n
   // Per-view constants, on the stack (no heap).
   DevCam dc[RAYGS_MAX_VIEWS];
   int64_t tiles = 0, trows = 0, pixels = 0;
-  int max_tx = 0;
-  if (!plan_views(cams, n_views, cfg, dc, tiles, trows, pixels, max_tx)) return RAYGS_ERR_INVALID_ARG;
+  int max_tx = 0, max_rows = 0;
+  if (!plan_views(cams, n_views, cfg, dc, tiles, trows, pixels, max_tx, max_rows)) return RAYGS_ERR_INVALID_ARG;
   if (cams[0].mip == RAYGS_MIP_EXACT) return RAYGS_ERR_INVALID_ARG;  // needs the second record buffer
 
   void *scratch = nullptr;
@@ -80,16 +80,17 @@ extern "C" raygs_status raygs_render_noalloc(const raygs_camera *cams, int32_t n
   w.tiles = tiles;
   w.trows = trows;
   w.max_tiles_x = max_tx;
+  w.max_rows = max_rows;
   w.num_sms = sms;
   w.G = sort_grid(sms);
   w.cfg = cfg;
-  const Layout L0 = make_layout(n_views, n, tiles, trows, 0, w.G, max_tx, false, false);
+  const Layout L0 = make_layout(n_views, n, tiles, trows, 0, w.G, max_tx, max_rows, false, false);
   if (L0.total + 8192 > kNoAllocScratchBytes) return RAYGS_ERR_CAPACITY;
   int64_t cap = int64_t((kNoAllocScratchBytes - L0.total - 8192) / (kBytesPerCapacity + 1));
-  w.L = make_layout(n_views, n, tiles, trows, cap, w.G, max_tx, false, false);
+  w.L = make_layout(n_views, n, tiles, trows, cap, w.G, max_tx, max_rows, false, false);
   while (w.L.total > kNoAllocScratchBytes && cap > 0) {
     cap -= 4096;
-    w.L = make_layout(n_views, n, tiles, trows, cap, w.G, max_tx, false, false);
+    w.L = make_layout(n_views, n, tiles, trows, cap, w.G, max_tx, max_rows, false, false);
   }
   if (cap <= 0 || w.L.total > kNoAllocScratchBytes) return RAYGS_ERR_CAPACITY;
   w.cap = cap;

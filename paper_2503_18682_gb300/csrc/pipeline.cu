@@ -72,14 +72,8 @@ int sort_grid(int num_sms) {
   return g > 1024 ? 1024 : (g < 1 ? 1 : g);
 }
 
-int tile_sort_bits(int64_t tiles) {
-  int b = 1;
-  while (b < 32 && (int64_t(1) << b) < tiles) ++b;
-  return b;
-}
-
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int G, int max_tiles_x,
-                   bool backward, bool mip_exact) {
+                   int max_rows, bool backward, bool mip_exact) {
   Layout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = up256(o + bytes); return r; };
@@ -89,34 +83,37 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.counters = take(sizeof(Counters));
   L.evals = take(4 * sizeof(unsigned long long));
   L.tilectr = take(16);
-  L.tscan = take(2 * sizeof(unsigned long long));
   L.depth = take(4 * VN);
   L.rect = take(8 * VN);
-  L.tcnt = take(VN);
+  L.rinfo = take(2 * VN);
   L.ell = take(sizeof(Ell) * VN);
   L.rec = take(sizeof(Rec) * VN);
   L.recx = mip_exact ? take(sizeof(Rec) * VN) : 0;
   for (int i = 0; i < 2; ++i) { L.s1k[i] = take(4 * VN); L.s1v[i] = take(4 * VN); }
-  L.off = take(4 * VN);
-  L.partial = take(4 * size_t(G));
-  L.rtstart_len = uint32_t(C / kEmitTile + 2);
-  L.rtstart = take(4 * size_t(L.rtstart_len));
+  L.vpos = n_views > 1 ? take(4 * VN) : 0;
+  const uint64_t pchunks = place_max_chunks(n_views, VN, max_rows);
+  L.cnt1 = take(4 * size_t(max_rows) * pchunks + 16);
   // per unit of capacity: kBytesPerCapacity bytes
-  L.seg = take(8 * C + 16);
-  L.seg_len = take(4 * C + 16);
-  L.seg_off = take(4 * C + 16);
-  for (int i = 0; i < 2; ++i) { L.rk[i] = take(4 * C + 16); L.rv[i] = take(8 * C + 16); }
+  L.spanl = take(4 * size_t(span_list_cap(C)));
+  L.spans = take(4 * size_t(span_rows_cap(C)));
+  L.rows = take(8 * C + 16);
   L.inst = take(4 * C + 16);
+  L.re = backward ? take(8 * C + 16) : 0;
+  L.inste = backward ? take(4 * C + 16) : 0;
+  L.ebase = backward ? take(4 * pchunks + 16) : 0;
+  L.paire = backward ? take(16 * VN + 16) : 0;
+  L.trcnt = take(4 * size_t(trows) + 16);
   L.trange = take(8 * size_t(trows) + 16);
   L.trinst = take(8 * size_t(trows) + 16);
   const int chunk_rows = expand_chunk_rows(cap, max_tiles_x);
   const int64_t max_chunks = expand_max_chunks(trows, cap, chunk_rows);
   L.cbase = take(4 * size_t(trows + 1) + 16);
   L.ccnt = take(4 * size_t(max_chunks) * size_t(max_tiles_x > 0 ? max_tiles_x : 1) + 16);
-  L.hist = take(4 * 512 * size_t(G) + 4 * (512 * size_t(G) / 2048 + 1));
+  L.hist = take(4 * 256 * size_t(G));
+  L.dtot = take(4 * 256);
   L.ranges = take(8 * size_t(tiles));
   L.tstop = take(4 * size_t(tiles) + 16);
-  L.deg = take(4 * VN);
+  L.deg = L.s1k[0];  // the FP64 lists of the vertex stage and of the backward: free then
   L.degc = take(4);
   L.partials = backward ? take(4 * kGradW * C + 16) : 0;
   L.pg = backward ? take(4 * kGradW * VN + 16) : 0;
@@ -125,8 +122,8 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
 }
 
 bool plan_views(const raygs_camera *cams, int n_views, const raygs_config &cfg, DevCam *dc, int64_t &tiles,
-                int64_t &trows, int64_t &pixels, int &max_tiles_x) {
-  tiles = 0; trows = 0; pixels = 0; max_tiles_x = 0;
+                int64_t &trows, int64_t &pixels, int &max_tiles_x, int &max_rows) {
+  tiles = 0; trows = 0; pixels = 0; max_tiles_x = 0; max_rows = 0;
   for (int v = 0; v < n_views; ++v) {
     if (!camera_valid(cams[v])) return false;
     if (cfg.divergence == 1 && cams[v].mip) return false;  // Eq. mip is a RayGS term
@@ -141,6 +138,7 @@ bool plan_views(const raygs_camera *cams, int n_views, const raygs_config &cfg, 
     trows += dc[v].tiles_y;
     pixels += int64_t(cams[v].width) * cams[v].height;
     if (dc[v].tiles_x > max_tiles_x) max_tiles_x = dc[v].tiles_x;
+    if (dc[v].tiles_y > max_rows) max_rows = dc[v].tiles_y;
     if (tiles >= (int64_t(1) << 31)) return false;
   }
   return true;
@@ -171,11 +169,14 @@ cudaError_t run_preprocess(Work &w, const raygs_scene &scene, cudaStream_t st) {
   P.tile_h = w.cfg.tile_h;
   P.depth_key = w.at<uint32_t>(w.L.depth);
   P.rect = w.at<uint2>(w.L.rect);
-  P.trow_cnt = w.at<uint8_t>(w.L.tcnt);
+  P.row_info = w.at<uint16_t>(w.L.rinfo);
   P.ell = w.at<Ell>(w.L.ell);
   P.rec = w.at<Rec>(w.L.rec);
   P.recx = w.L.recx ? w.at<Rec>(w.L.recx) : nullptr;
   P.counters = w.at<Counters>(w.L.counters);
+  P.span_list = w.at<uint32_t>(w.L.spanl);
+  P.span_list_cap = span_list_cap(uint64_t(w.cap));
+  P.span_cap = span_rows_cap(uint64_t(w.cap));
   P.deg_list = w.at<uint32_t>(w.L.deg);
   P.deg_count = w.at<uint32_t>(w.L.degc);
   return launch_preprocess(P, w.num_sms, st);
@@ -185,127 +186,89 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   Counters *ctr = w.at<Counters>(w.L.counters);
   const uint32_t VN = uint32_t(size_t(w.n_views) * size_t(w.n));
   const uint32_t cap = uint32_t(w.cap);
-  uint32_t *hist = w.at<uint32_t>(w.L.hist);
   cudaError_t e;
-  // 1. depth sort of the visible pairs: 4 passes of 8 bits over the float32 key; the values
-  // carry each pair's tile-row count above its id (bits of the largest id)
-  int id_bits = 1;
-  while (id_bits < 32 && (uint64_t(1) << id_bits) < uint64_t(VN)) ++id_bits;
+  SortPass base{};
+  base.hist = w.at<uint32_t>(w.L.hist);
+  base.digit_total = w.at<uint32_t>(w.L.dtot);
+  base.G = w.G;
+  base.count_max = VN;
+  base.n = uint32_t(w.n);
+  base.n_views = w.n_views;
+  // 1. depth sort of the visible pairs: 4 passes of 8 bits over the float32 key, which carry
+  // each pair's tile rows (the values' bits above those of the largest id, and the key's
+  // consumed digit)
+  base.id_bits = 1;
+  while (base.id_bits < 32 && (uint64_t(1) << base.id_bits) < uint64_t(VN)) ++base.id_bits;
   int cur = 0;
   for (int pass = 0; pass < 4; ++pass) {
-    SortPass sp{};
+    SortPass sp = base;
     sp.keys_in = w.at<uint32_t>(pass == 0 ? w.L.depth : w.L.s1k[cur]);
     sp.vals_in = pass == 0 ? nullptr : w.at<uint32_t>(w.L.s1v[cur]);
     const int dst = pass == 0 ? 0 : 1 - cur;
     sp.keys_out = w.at<uint32_t>(w.L.s1k[dst]);
     sp.vals_out = w.at<uint32_t>(w.L.s1v[dst]);
     sp.d_count = pass == 0 ? nullptr : &ctr->n_visible;
-    sp.count_max = VN;
     sp.shift = 8 * pass;
-    sp.bits = 8;
-    sp.filter = pass == 0 ? 1 : 0;
-    sp.hist = hist;
-    sp.G = w.G;
     sp.d_total = pass == 0 ? &ctr->n_visible : nullptr;
-    sp.row_cnt8 = pass == 0 ? w.at<uint8_t>(w.L.tcnt) : nullptr;
-    sp.id_bits = id_bits;
+    sp.row_info = pass == 0 ? w.at<uint16_t>(w.L.rinfo) : nullptr;
     sp.row_rect = pass == 3 ? w.at<uint2>(w.L.rect) : nullptr;
     if ((e = launch_sort_pass(sp, st)) != cudaSuccess) return e;
     cur = dst;
   }
   w.s1_final = cur;
-  const uint32_t *pairs = w.at<uint32_t>(w.L.s1v[cur]);
-  // 2a. pairs -> tile rows
-  ScanJob J{};
-  J.cnt = w.at<uint32_t>(w.L.s1k[cur]);  // the last depth pass left each pair's row count here
-  J.off = w.at<uint32_t>(w.L.off);
-  J.d_n = &ctr->n_visible;
-  J.partial = w.at<uint32_t>(w.L.partial);
-  J.tile_start = w.at<uint32_t>(w.L.rtstart);
-  J.tstart_len = w.L.rtstart_len;
-  J.d_total = &ctr->n_rows;
-  J.d_total_clamped = &ctr->n_rows_clamped;
-  J.cap = cap;
-  J.d_overflow = &ctr->overflow;
-  if ((e = launch_scan(J, w.G, st)) != cudaSuccess) return e;
-  // 2b. rows -> tile spans inside the support ellipse
-  RowsParams R{};
-  R.pairs = pairs;
-  R.rect = w.at<uint2>(w.L.rect);
+  // 2. several views: the pairs view by view (stable), with their positions in the depth order;
+  // the other ping-pong buffer takes the result, the depth order stays
+  const bool split = w.n_views > 1;
+  if (split) {
+    SortPass sp = base;
+    sp.keys_in = w.at<uint32_t>(w.L.s1k[cur]);
+    sp.keys_out = w.at<uint32_t>(w.L.s1k[1 - cur]);
+    sp.vals_in = w.at<uint32_t>(w.L.s1v[cur]);
+    sp.vals_out = w.at<uint32_t>(w.L.s1v[1 - cur]);
+    sp.index_out = w.at<uint32_t>(w.L.vpos);
+    sp.d_count = &ctr->n_visible;
+    sp.shift = 24;
+    if ((e = launch_sort_pass(sp, st)) != cudaSuccess) return e;
+  }
+  // 3. support rows into per-tile-row lists
+  PlaceParams R{};
+  R.info = w.at<uint32_t>(w.L.s1k[split ? 1 - cur : cur]);
+  R.pos = split ? w.at<uint32_t>(w.L.vpos) : nullptr;
+  R.ids = w.at<uint32_t>(w.L.s1v[split ? 1 - cur : cur]);
+  R.view_count = split ? base.digit_total : nullptr;
   R.ell = w.at<Ell>(w.L.ell);
   R.rec = w.at<Rec>(w.L.rec);
-  R.row_off = J.off;
-  R.row_tstart = J.tile_start;
   R.cams = w.at<DevCam>(w.L.cams);
   R.counters = ctr;
   R.n = int(w.n);
+  R.n_views = w.n_views;
   R.tile_w = w.cfg.tile_w;
   R.tile_h = w.cfg.tile_h;
-  R.seg = w.at<uint2>(w.L.seg);
-  R.seg_len = w.cfg.enable_backward ? w.at<uint32_t>(w.L.seg_len) : nullptr;
-  R.row_key = w.at<uint32_t>(w.L.rk[0]);
-  R.trow_inst = w.at<unsigned long long>(w.L.trinst);
   R.trows = int(w.trows);
+  R.max_rows = w.max_rows;
+  R.cap = cap;
+  R.span_list = w.at<uint32_t>(w.L.spanl);
+  R.span_list_cap = span_list_cap(uint64_t(w.cap));
+  R.spans = w.at<uint32_t>(w.L.spans);
+  R.cnt1 = w.at<uint32_t>(w.L.cnt1);
+  R.trow_cnt = w.at<uint32_t>(w.L.trcnt);
   R.trow_ranges = w.at<uint2>(w.L.trange);
-  if ((e = cudaMemsetAsync(R.trow_inst, 0, sizeof(unsigned long long) * size_t(w.trows), st)) != cudaSuccess)
-    return e;
-  if ((e = cudaMemsetAsync(R.trow_ranges, 0, sizeof(uint2) * size_t(w.trows), st)) != cudaSuccess) return e;
-  if ((e = launch_rows(R, w.G, st)) != cudaSuccess) return e;
-  ScanJob J2{};
-  J2.cnt = R.seg_len;
-  J2.off = w.at<uint32_t>(w.L.seg_off);
-  J2.d_n = &ctr->n_rows_clamped;
-  J2.partial = w.at<uint32_t>(w.L.partial);
-  J2.tile_start = nullptr;
-  J2.tstart_len = 0;
-  J2.d_total = &ctr->n_instances;
-  J2.d_total_clamped = &ctr->n_inst_clamped;
-  J2.cap = cap;
-  J2.d_overflow = &ctr->overflow;
-  // the emission offsets only index the backward's partials
-  const bool emission = w.cfg.enable_backward != 0;
-  if (emission && (e = launch_scan(J2, w.G, st)) != cudaSuccess) return e;
-  // first instance of every tile row, the instance total and the capacity check
-  if ((e = launch_trow_scan(R.trow_inst, R.trow_ranges, int(w.trows), ctr, cap, st)) != cudaSuccess) return e;
-  // 3. stable sort of the non-empty rows by global tile row (at most 8-bit digits); the first
-  // pass drops the empty rows and reads each row's payload as the row pass wrote it
-  const int rbits = tile_sort_bits(w.trows);
-  const int rpasses = (rbits + 7) / 8;
-  // digits of equal width (at least 4 bits): the first pass scatters into fewer buckets
-  // (64 instead of 256 for 12-bit tile rows), so its output runs are longer
-  const int rdigit = std::max(4, (rbits + rpasses - 1) / rpasses);
-  cur = 0;
-  for (int pass = 0; pass < rpasses; ++pass) {
-    SortPass sp{};
-    sp.keys_in = w.at<uint32_t>(w.L.rk[pass == 0 ? 0 : cur]);
-    sp.vals_in = nullptr;
-    const int dst = pass == 0 ? 1 : 1 - cur;
-    // (the sorted keys themselves are not read after the last pass)
-    sp.keys_out = pass + 1 < rpasses ? w.at<uint32_t>(w.L.rk[dst]) : nullptr;
-    sp.vals_out = nullptr;
-    sp.d_count = pass == 0 ? &ctr->n_rows_clamped : &ctr->n_rows_kept;
-    sp.count_max = cap;
-    sp.shift = rdigit * pass;
-    sp.bits = rdigit;
-    sp.filter = pass == 0 ? 1 : 0;
-    sp.hist = hist;
-    sp.G = w.G;
-    sp.d_total = pass == 0 ? &ctr->n_rows_kept : nullptr;
-    sp.wide = 1;
-    sp.wvals_in = pass == 0 ? R.seg : w.at<uint2>(w.L.rv[cur]);
-    sp.wvals_out = w.at<uint2>(w.L.rv[dst]);
-    if ((e = launch_sort_pass(sp, st)) != cudaSuccess) return e;
-    cur = dst;
-  }
-  w.s2_rows = cur;
-  // 4. tile-row ranges of the sorted rows, instances per tile, tile offsets, lists
-  // (each tile row's range of sorted rows came from the tile-row scan above)
-  uint2 *trange = R.trow_ranges;
+  R.trow_inst = w.at<unsigned long long>(w.L.trinst);
+  R.rows = w.at<uint2>(w.L.rows);
+  const bool backward = w.cfg.enable_backward != 0;
+  R.row_e = backward ? w.at<uint2>(w.L.re) : nullptr;
+  R.e_base = backward ? w.at<uint32_t>(w.L.ebase) : nullptr;
+  R.pair_e = backward ? w.at<uint4>(w.L.paire) : nullptr;
+  if ((e = launch_place(R, w.num_sms, st)) != cudaSuccess) return e;
+  // 4. instances per tile, tile offsets, lists
   ExpandParams X{};
   X.cams = R.cams;
   X.n_views = w.n_views;
-  X.trow_ranges = trange;
-  X.rows = w.at<uint2>(w.L.rv[cur]);
+  X.trow_ranges = R.trow_ranges;
+  X.rows = R.rows;
+  X.row_e = R.row_e;
+  X.e_base = R.e_base;
+  X.inst_e = backward ? w.at<uint32_t>(w.L.inste) : nullptr;
   X.trow_base = R.trow_inst;
   X.ranges = w.at<uint2>(w.L.ranges);
   X.inst = w.at<uint32_t>(w.L.inst);
@@ -316,6 +279,7 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   X.trows = int(w.trows);
   X.max_tiles_x = w.max_tiles_x;
   X.max_chunks = int(expand_max_chunks(w.trows, w.cap, X.chunk_rows));
+  X.counters = ctr;
   return launch_expand(X, st);
 }
 
@@ -360,10 +324,8 @@ cudaError_t run_backward(const Work &w, const raygs_scene &scene, const float *T
   B.inst_vals = w.at<uint32_t>(w.L.inst);
   B.pairs = w.at<uint32_t>(w.L.s1v[w.s1_final]);
   B.rec = w.at<Rec>(w.L.rec);
-  B.rect = w.at<uint2>(w.L.rect);
-  B.row_off = w.at<uint32_t>(w.L.off);
-  B.seg = w.at<uint2>(w.L.seg);
-  B.seg_off = w.at<uint32_t>(w.L.seg_off);
+  B.inst_e = w.at<uint32_t>(w.L.inste);
+  B.cap = uint32_t(w.cap);
   B.t_stop = w.cfg.t_stop;
   B.alpha_max = w.cfg.alpha_max;
   B.Tf = T_final;
@@ -375,8 +337,9 @@ cudaError_t run_backward(const Work &w, const raygs_scene &scene, const float *T
   if (e != cudaSuccess) return e;
   PairGradParams Q{};
   Q.pairs = B.pairs;
-  Q.row_off = B.row_off;
-  Q.seg_off = B.seg_off;
+  Q.pair_e = w.at<uint4>(w.L.paire);
+  Q.e_base = w.at<uint32_t>(w.L.ebase);
+  Q.cap = B.cap;
   Q.counters = w.at<Counters>(w.L.counters);
   Q.partials = B.partials;
   Q.pg = w.at<float>(w.L.pg);

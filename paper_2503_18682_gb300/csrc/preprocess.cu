@@ -486,10 +486,11 @@ __device__ __forceinline__ void write_record_mipx(const PrepParams &P, int64_t i
   e.cy = v.hi + so.dc1;
   e.a = so.M00; e.b = so.M01; e.d = so.M11; e.det = so.det;
   P.ell[idx] = e;
-  // the rectangle also in its own compact array (the backward gathers it by pair), and its
-  // tile-row count in a byte that the first depth-sort pass reads in pair order
+  // the rectangle also in its own compact array (read in depth order where the sort's spare
+  // bits do not hold its tile rows), and its tile rows in two bytes that the first depth-sort
+  // pass reads in pair order
   P.rect[idx] = make_uint2(e.r0, e.r1);
-  P.trow_cnt[idx] = uint8_t(min(so.ty1 - so.ty0 + 1, 255));
+  P.row_info[idx] = uint16_t(min(so.ty0, 255) | (min(so.ty1 - so.ty0 + 1, 255) << 8));
   if (write_key) P.depth_key[idx] = __float_as_uint(z);
 }
 
@@ -512,11 +513,18 @@ __device__ __forceinline__ void write_record(const PrepParams &P, int64_t idx, c
   e.cx = u.hi + so.dc0;
   e.cy = v.hi + so.dc1;
   e.a = so.M00; e.b = so.M01; e.d = so.M11; e.det = so.det;
+  if (!(so.M00 > 0.f)) {  // listed, with a place for its rows' spans (see PlaceParams)
+    const uint32_t rows = uint32_t(so.ty1 - so.ty0 + 1);
+    const uint32_t base = atomicAdd(&P.counters->n_span_rows, rows);
+    const uint32_t i = atomicAdd(&P.counters->n_unbounded, 1u);
+    const bool room = i < P.span_list_cap && base < P.span_cap && rows <= P.span_cap - base;
+    if (i < P.span_list_cap) P.span_list[i] = room ? uint32_t(idx) : kCulled;
+    e.cx = __uint_as_float(room ? base : kCulled);
+  }
   P.ell[idx] = e;
-  // the rectangle also in its own compact array (the backward gathers it by pair), and its
-  // tile-row count in a byte that the first depth-sort pass reads in pair order
+  // the rectangle also in its own compact array, and its tile rows in two bytes (see above)
   P.rect[idx] = make_uint2(e.r0, e.r1);
-  P.trow_cnt[idx] = uint8_t(min(so.ty1 - so.ty0 + 1, 255));
+  P.row_info[idx] = uint16_t(min(so.ty0, 255) | (min(so.ty1 - so.ty0 + 1, 255) << 8));
   if (write_key) P.depth_key[idx] = __float_as_uint(z);
 }
 

@@ -51,17 +51,22 @@ struct Counters {
   unsigned long long n_rows;
   unsigned long long n_instances;
   unsigned long long n_nonfinite;
-  uint32_t n_fp64;          // (primitive, view) pairs recomputed in FP64
+  uint32_t n_partials;      // partial-sum slots handed out (plans with the backward)
   uint32_t n_rows_kept;     // support rows with at least one tile
+  uint32_t n_unbounded;     // pairs whose support is not a bounded ellipse, and their rows
+  uint32_t n_span_rows;
+  uint32_t n_scan;          // rows of those pairs that have to be tested tile by tile
+  uint32_t pad;
 };
 
 // Screen-space support of a (primitive, view), one 32-byte sector for the tile-row pass:
 // its tile rectangle (as in the rect array) and the ellipse of pixel centres p with
 // (p - c)^T [[a, b], [b, d]] (p - c) <= 1 that holds exactly the rays with D <= kappa (up to
 // rounding), det = ad - b^2.  a < 0 marks a support that is not a bounded ellipse in the
-// image (or is too ill-conditioned in float32): binning then bounds it tile by tile from
-// the pair's record; a = -2 keeps every tile of the rectangle (the exact anti-aliasing
-// records hold no conic).
+// image (or is too ill-conditioned in float32): binning then bounds its rows from the pair's
+// record (cx holds, as bits, the pair's first slot among the spans, kCulled when there was no
+// room: its rows then keep the whole rectangle); a = -2 keeps every tile of the rectangle (the
+// exact anti-aliasing records hold no conic).
 struct __align__(32) Ell {
   uint32_t r0, r1;  // tx0 | ty0 << 16, tx1 | ty1 << 16
   float cx, cy, a, b, d, det;
@@ -162,90 +167,85 @@ struct PrepParams {
   int tile_w, tile_h;
   uint32_t *depth_key;
   uint2 *rect;
-  uint8_t *trow_cnt;    // tile rows of each pair's rectangle, saturated at 255
+  uint16_t *row_info;   // first tile row (low byte) and tile rows of each pair's rectangle, each saturated at 255
   Ell *ell;
   Rec *rec;
   Rec *recx;            // second half of the exact anti-aliasing record (views with mip = 2)
   Counters *counters;
+  uint32_t *span_list;  // pairs whose support is not a bounded ellipse, and room for their rows
+  uint32_t span_list_cap, span_cap;
   uint32_t *deg_list;   // (view, primitive) pairs left to the FP64 kernel
   uint32_t *deg_count;
 };
 
 struct SortPass {
   const uint32_t *keys_in;
-  const uint32_t *vals_in;
-  uint32_t *keys_out;       // nullable: the pass writes only the values
+  const uint32_t *vals_in;  // null: the item's index is its value (first depth pass)
+  uint32_t *keys_out;
   uint32_t *vals_out;
+  uint32_t *index_out;      // the items' indices (the split by view; null otherwise)
   const uint32_t *d_count;  // device item count (nullable: count_max is used)
   uint32_t count_max;
   int shift;
-  int bits;                 // digit width of this pass (8 for item ids, 4-8 for support rows)
-  int filter;               // drop kCulled keys; value = item index
-  uint32_t *hist;           // [digits][G], then the digit totals
+  uint32_t *hist;           // [digits][G]
+  uint32_t *digit_total;    // [digits] items of each digit
   int G;
   uint32_t *d_total;        // receives the number of items kept (nullable)
-  // wide mode (tile-row sort of the support rows): 8-byte values (sorted pair position,
-  // first tile column | run length << 16), as the row pass writes them
-  int wide;
-  const uint2 *wvals_in;
-  uint2 *wvals_out;
-  // The depth sort carries each pair's tile-row count above its id: the first pass packs
-  // min(count, field) into the bits above id_bits (row_cnt8: the dense per-pair count,
-  // saturated at 255; a full field means "not known"), and the last pass (row_rect set)
-  // writes the count in place of the key (the keys are not needed after it) and the bare id
-  // as the value, taking the count from the pair's rectangle when the field was full.
+  // The depth sort carries each pair's tile rows: the first pass (row_info: per pair in pair
+  // order, first tile row and row count, a byte each, saturated at 255) puts the first tile
+  // row in the key's low byte, the digit it has consumed, and min(count, field) into the
+  // value's bits above id_bits (a full field or byte means "not known"); the last pass
+  // (row_rect set) writes first tile row | (count - 1) << 12 | view << 24 in place of the key
+  // and the bare id as the value, taking what is not known from the pair's rectangle.
   // id_bits = 32 leaves no field: every count comes from the rectangle.
-  const uint8_t *row_cnt8;
+  const uint16_t *row_info;
   int id_bits;
   const uint2 *row_rect;
+  uint32_t n;               // primitives per view (the last depth pass)
+  int n_views;              // views (the split by view)
 };
 
-// Exclusive scan of per-unit output counts, with the unit that holds the first output of
-// every block of kEmitTile outputs (load-balanced expansion).
-struct ScanJob {
-  const uint32_t *cnt;
-  uint32_t *off;
-  const uint32_t *d_n;      // number of units (device; nullable: n_static is used)
-  uint32_t n_static;
-  uint32_t *partial;        // [G]
-  uint32_t *tile_start;
-  uint32_t tstart_len;
-  unsigned long long *d_total;
-  uint32_t *d_total_clamped;
-  uint32_t cap;
-  uint32_t *d_overflow;
-};
-
-struct RowsParams {
-  const uint32_t *pairs;    // sorted pair ids
-  const uint2 *rect;
+// Support rows of the depth-sorted pairs (rows.cu).
+struct PlaceParams {
+  const uint32_t *info;        // tile rows of each sorted pair, view by view (see SortPass)
+  const uint32_t *pos;         // its position in the depth order (null: one view, the index itself)
+  const uint32_t *ids;         // its pair id
+  const uint32_t *view_count;  // pairs of each view (null: one view, all of them)
   const Ell *ell;
   const Rec *rec;
-  const uint32_t *row_off;
-  const uint32_t *row_tstart;
   const DevCam *cams;
-  const Counters *counters;
-  int n;                    // primitives per view
-  int tile_w, tile_h;
-  uint2 *seg;               // per row: (sorted pair position, txa | len << 16), len the tiles
-                            // of the row inside the support (the tile-row sort's payload)
-  uint32_t *seg_len;        // per row: len again, for the emission-offset scan (backward
-                            // plans only; nullable)
-  uint32_t *row_key;        // per row: global tile row, or kCulled when the run is empty
-  unsigned long long *trow_inst;  // [tile rows] instances of each tile row (accumulated)
-  uint2 *trow_ranges;             // [tile rows] .y: non-empty rows of each tile row (accumulated)
-  int trows;
+  Counters *counters;
+  int n, n_views, tile_w, tile_h;
+  int trows, max_rows;         // tile rows of the batch, and the most of one view
+  uint32_t cap;
+  uint32_t cp_lo, cp_hi, target;
+  const uint32_t *span_list;   // pairs whose support is not a bounded ellipse (see PrepParams)
+  uint32_t span_list_cap;
+  uint32_t *spans;             // per row of those pairs: first tile column | tiles << 16
+  uint32_t *cnt1;              // per view, tile row and chunk: rows, then rows of the chunks before
+  uint32_t *trow_cnt;          // [tile rows] rows
+  uint2 *trow_ranges;          // [tile rows] the tile row's range of the row list
+  unsigned long long *trow_inst;  // [tile rows] cleared here
+  uint2 *rows;                 // [cap] the row list: sorted pair position, first tile column | tiles << 16
+  // plans with the backward (null otherwise): where each row's instances lie among the partial
+  // sums, (chunk, offset in the chunk); the chunks' first slots; per sorted pair its run
+  // (first, end, chunk)
+  uint2 *row_e;
+  uint32_t *e_base;
+  uint4 *pair_e;
 };
-constexpr int kTrowsShared = 2048;  // tile rows whose totals a CTA keeps in shared memory
 
-// Per-tile-row passes over the support rows sorted by tile row (stable, so each tile row
-// lists its rows in depth order): per-tile instance counts, then the instance lists.
+// Per-tile-row passes over the support rows listed by tile row (in depth order): per-tile instance counts, then the instance lists.
 struct ExpandParams {
   const DevCam *cams;
   int n_views;
-  const uint2 *trow_ranges;  // [tile rows] range of the tile row in the sorted rows
-  const uint2 *rows;         // sorted rows: (sorted pair position, txa | len << 16)
-  const unsigned long long *trow_base;  // [tile rows] first instance of each tile row
+  const uint2 *trow_ranges;  // [tile rows] range of the tile row in the row list
+  const uint2 *rows;         // the row list (see PlaceParams)
+  const uint2 *row_e;
+  const uint32_t *e_base;
+  uint32_t *inst_e;          // [cap] partial-sum slot of every instance (plans with the backward)
+  unsigned long long *trow_base;  // [tile rows] instances of each tile row, then its first instance
+  Counters *counters;
   uint2 *ranges;             // [tiles] instance range of every tile (clamped to cap)
   uint32_t *inst;            // [cap] sorted pair position of every instance
   uint32_t cap;
@@ -280,7 +280,6 @@ struct RenderParams {
                         // stopped, or kCulled when the list ran out first (nullable)
 };
 
-constexpr int kEmitTile = 2048;
 constexpr int kMaxTilesX = 4096;  // tiles in one tile row (32768-pixel views at 8-pixel tiles)
 constexpr int kGradW = 13;  // per-instance / per-pair gradient partials (see backward.cu)
 
@@ -289,24 +288,23 @@ struct BackParams {
   int n_views;
   const uint2 *ranges;
   const uint32_t *inst_vals;
+  const uint32_t *inst_e;  // partial-sum slot of every instance
   const uint32_t *pairs;
   const Rec *rec;
-  const uint2 *rect;
-  const uint32_t *row_off;
-  const uint2 *seg;
-  const uint32_t *seg_off;
+  uint32_t cap;
   float t_stop, alpha_max;
   const float *Tf;
   const int *ncontrib;
   const float *dL_drgb;
   const float *dL_dT;   // nullable
-  float *partials;      // [capacity][kGradW] by emission index
+  float *partials;      // [capacity][kGradW] by partial-sum slot
 };
 
 struct PairGradParams {
   const uint32_t *pairs;
-  const uint32_t *row_off;
-  const uint32_t *seg_off;
+  const uint4 *pair_e;     // per sorted pair: its run of partial sums (first, end, chunk)
+  const uint32_t *e_base;
+  uint32_t cap;
   const Counters *counters;
   const float *partials;
   float *pg;            // [V*N][kGradW] by pair id
@@ -336,10 +334,9 @@ void note_cuda_error(cudaError_t e);
 
 cudaError_t launch_preprocess(const PrepParams &P, int num_sms, cudaStream_t st);
 cudaError_t launch_sort_pass(SortPass p, cudaStream_t st);
-cudaError_t launch_scan(const ScanJob &J, int G, cudaStream_t st);
-cudaError_t launch_rows(const RowsParams &R, int G, cudaStream_t st);
-cudaError_t launch_trow_scan(unsigned long long *trow_inst, uint2 *trow_ranges, int trows, Counters *c, uint32_t cap,
-                             cudaStream_t st);
+uint32_t place_cp_lo(int max_rows);
+uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows);
+cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st);
 cudaError_t launch_expand(const ExpandParams &E, cudaStream_t st);
 int expand_chunk_rows(int64_t cap, int max_tiles_x);
 int64_t expand_max_chunks(int64_t trows, int64_t cap, int chunk_rows);
@@ -356,16 +353,19 @@ cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo
 // ---------------------------------------------------------------- workspace
 // Byte offsets of every buffer inside one caller-owned (or library-static) workspace.
 struct Layout {
-  size_t tilectr, cams, counters, evals, tstop, tscan, depth, rect, tcnt, ell, rec, recx, s1k[2], s1v[2], off, partial, rtstart,
-      seg, seg_len, seg_off, rk[2], rv[2], trange, trinst, cbase, ccnt, inst, hist, ranges, deg, degc, partials, pg, total;
-  uint32_t rtstart_len;
+  size_t tilectr, cams, spanl, spans, vpos, counters, evals, tstop, depth, rect, rinfo, ell, rec, recx, s1k[2], s1v[2], cnt1, trcnt, rows,
+      re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, pg, total;
 };
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int G, int max_tiles_x,
-                   bool backward, bool mip_exact);
+                   int max_rows, bool backward, bool mip_exact);
 
-// Workspace bytes per unit of instance capacity (tile rows and instances share it).
-constexpr size_t kBytesPerCapacity = 8 + 4 + 4 + 2 * 4 + 2 * 8 + 4;
+// Workspace bytes per unit of instance capacity (support rows and instances share it).
+constexpr size_t kBytesPerCapacity = 8 + 4 + 1;
+// Room for the pairs whose support is not a bounded ellipse and for their rows' spans (2 % of
+// the rows on the stereo batch, whose cameras stand among the primitives).
+constexpr uint32_t span_list_cap(uint64_t cap) { return uint32_t(cap / 32) + 256; }
+constexpr uint32_t span_rows_cap(uint64_t cap) { return uint32_t(cap / 8) + 1024; }
 
 // A bound workspace and the sizes it was laid out for.
 struct Work {
@@ -373,10 +373,10 @@ struct Work {
   Layout L{};
   int n_views = 0;
   int64_t n = 0, tiles = 0, trows = 0, cap = 0;
-  int max_tiles_x = 0;
+  int max_tiles_x = 0, max_rows = 0;  // most tile columns and rows of one view
   int G = 0, num_sms = 0;
   raygs_config cfg{};
-  int s1_final = 0, s2_rows = 0;  // which ping-pong buffers hold the sorted results
+  int s1_final = 0;  // which ping-pong buffer holds the depth-sorted pairs
   template <typename T>
   T *at(size_t off) const { return reinterpret_cast<T *>(base + off); }
 };
@@ -386,13 +386,12 @@ void fill_devcam(const raygs_camera &c, const raygs_config &cfg, DevCam &d);
 // Per-view constants and the global tile, tile-row and pixel numbering of a batch of views;
 // false when a view is invalid or the batch is too large to number in 31 bits.
 bool plan_views(const raygs_camera *cams, int n_views, const raygs_config &cfg, DevCam *dc, int64_t &tiles,
-                int64_t &trows, int64_t &pixels, int &max_tiles_x);
+                int64_t &trows, int64_t &pixels, int &max_tiles_x, int &max_rows);
 bool config_valid(const raygs_config &cfg);
 bool camera_valid(const raygs_camera &c);
 raygs_status scene_valid(const raygs_scene *s, int64_t n);
 
 int sort_grid(int num_sms);
-int tile_sort_bits(int64_t tiles);
 cudaError_t run_preprocess(Work &w, const raygs_scene &scene, cudaStream_t st);
 cudaError_t run_bin_sort(Work &w, cudaStream_t st);
 cudaError_t run_render(const Work &w, float *rgb, float *T_final, int32_t *n_contrib, bool count,
