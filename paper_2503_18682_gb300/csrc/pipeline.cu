@@ -72,7 +72,7 @@ int sort_grid(int num_sms) {
   return g > 1024 ? 1024 : (g < 1 ? 1 : g);
 }
 
-Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int G, int max_tiles_x,
+Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
                    int max_rows, bool backward, bool mip_exact) {
   Layout L{};
   size_t o = 0;
@@ -105,11 +105,9 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.trcnt = take(4 * size_t(trows) + 16);
   L.trange = take(8 * size_t(trows) + 16);
   L.trinst = take(8 * size_t(trows) + 16);
-  const int chunk_rows = expand_chunk_rows(cap, max_tiles_x);
-  const int64_t max_chunks = expand_max_chunks(trows, cap, chunk_rows);
   L.cbase = take(4 * size_t(trows + 1) + 16);
-  L.ccnt = take(4 * size_t(max_chunks) * size_t(max_tiles_x > 0 ? max_tiles_x : 1) + 16);
-  L.hist = take(4 * 256 * size_t(G));
+  L.ccnt = take(4 * size_t(list_max_chunks(trows, cap, max_tiles_x, num_sms)) * size_t(max_tiles_x) + 16);
+  L.hist = take(4 * 256 * size_t(sort_grid(num_sms)));
   L.dtot = take(4 * 256);
   L.ranges = take(8 * size_t(tiles));
   L.tstop = take(4 * size_t(tiles) + 16);
@@ -255,32 +253,35 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   R.trow_ranges = w.at<uint2>(w.L.trange);
   R.trow_inst = w.at<unsigned long long>(w.L.trinst);
   R.rows = w.at<uint2>(w.L.rows);
+  R.chunk_base = w.at<uint32_t>(w.L.cbase);
+  R.list_hi = list_rows_hi(w.cap, w.max_tiles_x);
+  R.list_target = list_target(w.num_sms);
+  R.max_chunks = uint32_t(list_max_chunks(w.trows, w.cap, w.max_tiles_x, w.num_sms));
   const bool backward = w.cfg.enable_backward != 0;
   R.row_e = backward ? w.at<uint2>(w.L.re) : nullptr;
   R.e_base = backward ? w.at<uint32_t>(w.L.ebase) : nullptr;
   R.pair_e = backward ? w.at<uint4>(w.L.paire) : nullptr;
   if ((e = launch_place(R, w.num_sms, st)) != cudaSuccess) return e;
   // 4. instances per tile, tile offsets, lists
-  ExpandParams X{};
+  ListParams X{};
   X.cams = R.cams;
   X.n_views = w.n_views;
+  X.counters = ctr;
   X.trow_ranges = R.trow_ranges;
   X.rows = R.rows;
   X.row_e = R.row_e;
   X.e_base = R.e_base;
   X.inst_e = backward ? w.at<uint32_t>(w.L.inste) : nullptr;
-  X.trow_base = R.trow_inst;
+  X.trow_inst = R.trow_inst;
   X.ranges = w.at<uint2>(w.L.ranges);
   X.inst = w.at<uint32_t>(w.L.inst);
   X.cap = cap;
-  X.chunk_base = w.at<uint32_t>(w.L.cbase);
-  X.chunk_cnt = w.at<uint32_t>(w.L.ccnt);
-  X.chunk_rows = expand_chunk_rows(w.cap, w.max_tiles_x);
+  X.chunk_base = R.chunk_base;
+  X.cnt2 = w.at<uint32_t>(w.L.ccnt);
   X.trows = int(w.trows);
   X.max_tiles_x = w.max_tiles_x;
-  X.max_chunks = int(expand_max_chunks(w.trows, w.cap, X.chunk_rows));
-  X.counters = ctr;
-  return launch_expand(X, st);
+  X.max_chunks = R.max_chunks;
+  return launch_lists(X, w.num_sms, st);
 }
 
 cudaError_t run_render(const Work &w, float *rgb, float *T_final, int32_t *n_contrib, bool count,

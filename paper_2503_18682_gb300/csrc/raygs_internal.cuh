@@ -56,6 +56,8 @@ struct Counters {
   uint32_t n_unbounded;     // pairs whose support is not a bounded ellipse, and their rows
   uint32_t n_span_rows;
   uint32_t n_scan;          // rows of those pairs that have to be tested tile by tile
+  uint32_t chunk_rows;      // rows per chunk of the list pass
+  uint32_t lists_done;      // CTAs of list_count_kernel that have finished (0 between launches)
   uint32_t pad;
 };
 
@@ -226,6 +228,8 @@ struct PlaceParams {
   uint32_t *trow_cnt;          // [tile rows] rows
   uint2 *trow_ranges;          // [tile rows] the tile row's range of the row list
   unsigned long long *trow_inst;  // [tile rows] cleared here
+  uint32_t *chunk_base;        // [tile rows + 1] first chunk of each tile row in the list pass
+  uint32_t list_hi, list_target, max_chunks;
   uint2 *rows;                 // [cap] the row list: sorted pair position, first tile column | tiles << 16
   // plans with the backward (null otherwise): where each row's instances lie among the partial
   // sums, (chunk, offset in the chunk); the chunks' first slots; per sorted pair its run
@@ -235,27 +239,29 @@ struct PlaceParams {
   uint4 *pair_e;
 };
 
-// Per-tile-row passes over the support rows listed by tile row (in depth order): per-tile instance counts, then the instance lists.
-struct ExpandParams {
+// Instance lists from the support rows listed by tile row, in depth order (lists.cu).
+struct ListParams {
   const DevCam *cams;
   int n_views;
+  Counters *counters;
   const uint2 *trow_ranges;  // [tile rows] range of the tile row in the row list
   const uint2 *rows;         // the row list (see PlaceParams)
   const uint2 *row_e;
   const uint32_t *e_base;
   uint32_t *inst_e;          // [cap] partial-sum slot of every instance (plans with the backward)
-  unsigned long long *trow_base;  // [tile rows] instances of each tile row, then its first instance
-  Counters *counters;
+  unsigned long long *trow_inst;  // [tile rows] instances of each tile row, then its first instance
   uint2 *ranges;             // [tiles] instance range of every tile (clamped to cap)
   uint32_t *inst;            // [cap] sorted pair position of every instance
   uint32_t cap;
-  // Each tile row's sorted rows are cut into chunks of chunk_rows rows (at least one chunk
-  // per tile row), one CTA each: chunk_base[t] is tile row t's first chunk (chunk_base[trows]
-  // the number of chunks), chunk_cnt[chunk][x] the chunk's instances in tile column x.
-  uint32_t *chunk_base;
-  uint32_t *chunk_cnt;
-  int chunk_rows, trows, max_tiles_x, max_chunks;
+  // Each tile row's rows are cut into chunks (at least one): chunk_base[t] is tile row t's first
+  // chunk (chunk_base[trows] the number of chunks), cnt2[chunk][x] the chunk's instances in
+  // tile column x.
+  const uint32_t *chunk_base;
+  uint32_t *cnt2;
+  int trows, max_tiles_x;
+  uint32_t max_chunks;
 };
+constexpr uint32_t kListRowsLo = 512;  // rows of the shortest chunk
 
 struct RenderParams {
   const DevCam *cams;
@@ -337,9 +343,10 @@ cudaError_t launch_sort_pass(SortPass p, cudaStream_t st);
 uint32_t place_cp_lo(int max_rows);
 uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows);
 cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st);
-cudaError_t launch_expand(const ExpandParams &E, cudaStream_t st);
-int expand_chunk_rows(int64_t cap, int max_tiles_x);
-int64_t expand_max_chunks(int64_t trows, int64_t cap, int chunk_rows);
+uint32_t list_rows_hi(int64_t cap, int max_tiles_x);
+uint32_t list_target(int num_sms);
+uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sms);
+cudaError_t launch_lists(const ListParams &P, int num_sms, cudaStream_t st);
 cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int batch_records, int num_sms,
                           bool count, cudaStream_t st);
 cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int64_t n_tiles, bool count,
@@ -357,7 +364,7 @@ struct Layout {
       re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, pg, total;
 };
 
-Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int G, int max_tiles_x,
+Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
                    int max_rows, bool backward, bool mip_exact);
 
 // Workspace bytes per unit of instance capacity (support rows and instances share it).

@@ -433,7 +433,7 @@ __device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long lo
 
 // The tile rows' ranges in the row list (one CTA; 64-bit running sums, clamped to the
 // capacity: every slot below it belongs to exactly one row), the row total, the capacity
-// check, and the tile rows' instance totals cleared for the list pass.
+// check, the chunks of the list pass, and its instance totals cleared.
 __global__ void __launch_bounds__(1024) trow_plan_kernel(PlaceParams P) {
   __shared__ unsigned long long ws[33];
   const int per = (P.trows + 1023) / 1024;
@@ -447,6 +447,27 @@ __global__ void __launch_bounds__(1024) trow_plan_kernel(PlaceParams P) {
     P.trow_ranges[t] = make_uint2(uint32_t(min(run, cap)), uint32_t(min(run + n, cap)));
     P.trow_inst[t] = 0ull;
     run += n;
+  }
+  // the chunks of the list pass: the shortest power of two in [kListRowsLo, list_hi] that leaves
+  // fewer than list_target of them (short lists still occupy every SM), at least one per tile
+  // row (its tiles' ranges are written with them)
+  uint32_t cr = kListRowsLo;
+  while (cr < P.list_hi && uint32_t(min(tot, cap)) / cr >= P.list_target) cr <<= 1;
+  auto chunks = [&](int t) {
+    const uint2 rr = P.trow_ranges[t];  // (this thread wrote it)
+    return max(1u, (rr.y - rr.x + cr - 1) / cr);
+  };
+  s = 0;
+  for (int t = b; t < e; ++t) s += chunks(t);
+  unsigned long long nchunks;
+  run = block_excl_scan64(s, ws, &nchunks);
+  for (int t = b; t < e; ++t) {
+    P.chunk_base[t] = uint32_t(run);
+    run += chunks(t);
+  }
+  if (threadIdx.x == 0) {
+    P.chunk_base[P.trows] = uint32_t(min(nchunks, (unsigned long long)P.max_chunks));
+    P.counters->chunk_rows = cr;
   }
   if (threadIdx.x == 0) {
     P.counters->n_rows = tot;
