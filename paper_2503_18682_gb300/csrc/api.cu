@@ -98,7 +98,7 @@ raygs_status raygs_plan_create(const raygs_camera *cams, int32_t n_views, int64_
   w.G = sort_grid(sms);
   w.cfg = cfg;
   w.L = make_layout(n_views, n_gaussians, tb, trows, max_instances, sms, max_tx, max_rows, cfg.enable_backward != 0,
-                    cams[0].mip == RAYGS_MIP_EXACT);
+                    cams[0].mip == RAYGS_MIP_EXACT, true);
   p->total_pixels = pb;
   *out = p;
   return RAYGS_OK;
@@ -120,7 +120,7 @@ raygs_status raygs_plan_bind(raygs_plan *plan, void *workspace, size_t bytes) {
   cudaError_t e = cudaMemcpy(plan->w.base + plan->w.L.cams, plan->dcams.data(),
                              sizeof(DevCam) * plan->w.n_views, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(e);
-  e = cudaMemset(plan->w.base + plan->w.L.counters, 0, sizeof(Counters));
+  e = cudaMemset(plan->w.base + plan->w.L.counters, 0, sizeof(Counters) + 16);
   if (e != cudaSuccess) return cuda_fail(e);
   plan->stage = 0;
   return RAYGS_OK;

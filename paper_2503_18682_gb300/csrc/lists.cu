@@ -197,7 +197,14 @@ __global__ void __launch_bounds__(NT) list_kernel(ListParams P) {
     for (int x = x0; x < x1; ++x) {
       const uint32_t n = s_tot[x];
       s_cur[x] = o + s_bef[x];
-      if (chunk_c == 0) P.ranges[tile0 + x] = make_uint2(min(o, P.cap), min(o + n, P.cap));
+      if (chunk_c == 0) {
+        const uint2 r = make_uint2(min(o, P.cap), min(o + n, P.cap));
+        P.ranges[tile0 + x] = r;
+        if (P.class_tiles) {
+          const int c = tile_class_of(r.y - r.x);
+          P.class_tiles[size_t(c) * size_t(P.tiles) + atomicAdd(&P.counters->tile_class[c], 1u)] = tile0 + x;
+        }
+      }
       o += n;
     }
   }

@@ -73,16 +73,16 @@ int sort_grid(int num_sms) {
 }
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
-                   int max_rows, bool backward, bool mip_exact) {
+                   int max_rows, bool backward, bool mip_exact, bool tile_order) {
   Layout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = up256(o + bytes); return r; };
   const size_t VN = size_t(n_views) * size_t(n);
   const size_t C = size_t(cap);
   L.cams = take(sizeof(DevCam) * size_t(n_views));
-  L.counters = take(sizeof(Counters));
+  L.counters = take(sizeof(Counters) + 16);  // and the rasteriser's tile counter
+  L.tilectr = L.counters + sizeof(Counters);
   L.evals = take(4 * sizeof(unsigned long long));
-  L.tilectr = take(16);
   L.depth = take(4 * VN);
   L.rect = take(8 * VN);
   L.rinfo = take(2 * VN);
@@ -110,6 +110,7 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.hist = take(4 * 256 * size_t(sort_grid(num_sms)));
   L.dtot = take(4 * 256);
   L.ranges = take(8 * size_t(tiles));
+  L.tclass = tile_order ? take(4 * size_t(kTileClasses) * size_t(tiles) + 16) : 0;
   L.tstop = take(4 * size_t(tiles) + 16);
   L.deg = L.s1k[0];  // the FP64 lists of the vertex stage and of the backward: free then
   L.degc = take(4);
@@ -143,7 +144,7 @@ bool plan_views(const raygs_camera *cams, int n_views, const raygs_config &cfg, 
 }
 
 cudaError_t run_preprocess(Work &w, const raygs_scene &scene, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(w.base + w.L.counters, 0, sizeof(Counters), st);
+  cudaError_t e = cudaMemsetAsync(w.base + w.L.counters, 0, sizeof(Counters) + 16, st);
   if (e != cudaSuccess) return e;
   PrepParams P{};
   P.means = scene.means;
@@ -274,6 +275,8 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   X.inst_e = backward ? w.at<uint32_t>(w.L.inste) : nullptr;
   X.trow_inst = R.trow_inst;
   X.ranges = w.at<uint2>(w.L.ranges);
+  X.class_tiles = w.L.tclass ? w.at<uint32_t>(w.L.tclass) : nullptr;
+  X.tiles = w.tiles;
   X.inst = w.at<uint32_t>(w.L.inst);
   X.cap = cap;
   X.chunk_base = R.chunk_base;
@@ -307,12 +310,12 @@ cudaError_t run_render(const Work &w, float *rgb, float *T_final, int32_t *n_con
     cudaError_t e = cudaMemsetAsync(P.eval_counts, 0, 4 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
   }
-  if (P.recx) return launch_render_mipx(P, w.cfg.tile_w, w.cfg.tile_h, w.tiles, count, st);
   if (w.tiles == 0) return cudaSuccess;
   P.tile_counter = w.at<unsigned int>(w.L.tilectr);
   P.n_tiles = int(w.tiles);
-  cudaError_t e = cudaMemsetAsync(P.tile_counter, 0, sizeof(unsigned int), st);
-  if (e != cudaSuccess) return e;
+  P.counters = w.at<Counters>(w.L.counters);
+  P.class_tiles = w.L.tclass ? w.at<uint32_t>(w.L.tclass) : nullptr;
+  if (P.recx) return launch_render_mipx(P, w.cfg.tile_w, w.cfg.tile_h, w.num_sms, count, st);
   return launch_render(P, w.cfg.tile_w, w.cfg.tile_h, w.cfg.batch_records, w.num_sms, count, st);
 }
 

@@ -58,8 +58,22 @@ struct Counters {
   uint32_t n_scan;          // rows of those pairs that have to be tested tile by tile
   uint32_t chunk_rows;      // rows per chunk of the list pass
   uint32_t lists_done;      // CTAs of list_count_kernel that have finished (0 between launches)
-  uint32_t pad;
+  uint32_t tile_class[16];                    // tiles of each class (see tile_class_of)
 };
+
+// Classes of tiles by list length, longest first: the rasteriser takes them in this order (a
+// tile with a long list started last would run alone at the end).
+constexpr int kTileClasses = 12;
+__host__ __device__ constexpr uint32_t tile_class_min(int c) {
+  constexpr uint32_t m[kTileClasses] = {4096, 2048, 1024, 768, 512, 384, 256, 192, 128, 64, 16, 0};
+  return m[c];
+}
+__device__ __forceinline__ int tile_class_of(uint32_t len) {
+  int c = 0;
+#pragma unroll
+  for (int k = 0; k < kTileClasses - 1; ++k) c += len < tile_class_min(k) ? 1 : 0;
+  return c;
+}
 
 // Screen-space support of a (primitive, view), one 32-byte sector for the tile-row pass:
 // its tile rectangle (as in the rect array) and the ellipse of pixel centres p with
@@ -251,6 +265,8 @@ struct ListParams {
   uint32_t *inst_e;          // [cap] partial-sum slot of every instance (plans with the backward)
   unsigned long long *trow_inst;  // [tile rows] instances of each tile row, then its first instance
   uint2 *ranges;             // [tiles] instance range of every tile (clamped to cap)
+  uint32_t *class_tiles;     // [kTileClasses][tiles] the tiles of each class (nullable)
+  int64_t tiles;
   uint32_t *inst;            // [cap] sorted pair position of every instance
   uint32_t cap;
   // Each tile row's rows are cut into chunks (at least one): chunk_base[t] is tile row t's first
@@ -272,8 +288,12 @@ struct RenderParams {
   const Rec *rec;
   float t_stop, alpha_max;
   float qmix;  // 1: D_ray fragment formula, D ~ q / (q + r); 0: D_gs, D ~ q (records with h = 0)
-  unsigned int *tile_counter;  // next unclaimed tile of the persistent rasteriser (zeroed per launch)
+  unsigned int *tile_counter;  // [0] next unclaimed item of the persistent rasteriser, [1] CTAs that
+                               // have left it; both 0 between launches (the last CTA clears them)
   int n_tiles;
+  const Counters *counters;
+  const uint32_t *class_tiles;  // tiles by class (nullable: tile order)
+  int slots;                    // CTAs resident at a time (set at the launch)
   const Rec *recx;  // exact anti-aliasing: second half of each record (then rec holds the first)
   float p_min;
   float *rgb;
@@ -349,7 +369,7 @@ uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sm
 cudaError_t launch_lists(const ListParams &P, int num_sms, cudaStream_t st);
 cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int batch_records, int num_sms,
                           bool count, cudaStream_t st);
-cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int64_t n_tiles, bool count,
+cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int num_sms, bool count,
                                cudaStream_t st);
 cudaError_t launch_render_backward(const BackParams &P, int tile_w, int tile_h, int64_t n_tiles, cudaStream_t st);
 cudaError_t launch_pair_grads(const PairGradParams &P, int G, cudaStream_t st);
@@ -360,12 +380,12 @@ cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo
 // ---------------------------------------------------------------- workspace
 // Byte offsets of every buffer inside one caller-owned (or library-static) workspace.
 struct Layout {
-  size_t tilectr, cams, spanl, spans, vpos, counters, evals, tstop, depth, rect, rinfo, ell, rec, recx, s1k[2], s1v[2], cnt1, trcnt, rows,
+  size_t tilectr, tclass, cams, spanl, spans, vpos, counters, evals, tstop, depth, rect, rinfo, ell, rec, recx, s1k[2], s1v[2], cnt1, trcnt, rows,
       re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, pg, total;
 };
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
-                   int max_rows, bool backward, bool mip_exact);
+                   int max_rows, bool backward, bool mip_exact, bool tile_order);
 
 // Workspace bytes per unit of instance capacity (support rows and instances share it).
 constexpr size_t kBytesPerCapacity = 8 + 4 + 1;

@@ -2,7 +2,7 @@
 // Eq. rend_opacity; Sec. 4.2 fragment formula).
 //
 // Persistent CTAs (one per resident slot) claim the screen tiles of all views from a
-// counter, one at a time; each thread shades PX pixels of a tile row.  A tile's instance list (depth order) is consumed in batches: each thread
+// counter, one at a time, those with the longest lists first; each thread shades PX pixels of a tile row.  A tile's instance list (depth order) is consumed in batches: each thread
 // stages records in shared memory, converting the projected centre to a tile-relative
 // offset in double-float so that per-pixel offsets stay exact to the float32 rounding of
 // the offset itself.  Per pixel, with delta = pixel centre - projected centre:
@@ -25,195 +25,270 @@
 
 namespace raygs {
 
-template <int TW, int TH, int PX, int NBF, bool COUNT, int DIV>
-__global__ void __launch_bounds__(TW *TH / PX, 16) render_kernel(RenderParams P) {
-  constexpr int NT = TW * TH / PX;  // threads
-  constexpr int NB = NBF * NT;      // records per batch
-  constexpr int QX = TW / PX;       // threads per tile row
-  __shared__ float4 s_A[NB], s_B[NB], s_C[NB], s_D[NB];
-  __shared__ Rec s_raw[NB];
-  __shared__ int s_view, s_tile;
-  const int tid = threadIdx.x;
-  // persistent CTAs: each claims the next tile until none is left
-  for (;;) {
-  if (tid == 0) s_tile = int(atomicAdd(P.tile_counter, 1u));
-  __syncthreads();
-  const int tile = s_tile;
-  if (tile >= P.n_tiles) break;
-  if (tid == 0) {
-    int v = 0;
-    while (v + 1 < P.n_views && P.cams[v + 1].tile_base <= tile) ++v;
-    s_view = v;
-  }
-  __syncthreads();
-  const DevCam &cam = P.cams[s_view];
-  const int local = tile - cam.tile_base;
-  const int ty = local / cam.tiles_x, tx = local - ty * cam.tiles_x;
-  const int px0 = tx * TW, py0 = ty * TH;
-  const int lx = tid % QX, ly = tid / QX;
-  const int px = px0 + lx, py = py0 + ly;
-  const uint2 rg = P.ranges[tile];
-  const float ox_tile = float(px0) + 0.5f, oy_tile = float(py0) + 0.5f;
-  const float fl_x = float(lx), fl_y = float(ly), step = float(QX);
-
+// Compositing state of a thread's pixels.
+template <int PX>
+struct Pixels {
   float T[PX], C0[PX], C1[PX], C2[PX];
   int last[PX];
-  uint32_t alive = 0;
-#pragma unroll
-  for (int k = 0; k < PX; ++k) {
-    T[k] = 1.f; C0[k] = 0.f; C1[k] = 0.f; C2[k] = 0.f; last[k] = 0;
-    if (py < cam.H && px + k * QX < cam.W) alive |= 1u << k;
-  }
-  const uint32_t inside = alive;
-  unsigned long long n_eval = 0, n_comp = 0, n_iter = 0;
-  uint32_t stop_at = rg.y;  // first list entry the CTA did not stage
+  uint32_t alive;
+  unsigned long long n_eval, n_comp, n_iter;  // instrumented variant
+};
 
-  // Records move through a two-stage pipeline: while a batch is composited, the raw
-  // records of the next batch are in flight to shared memory (cp.async) and the record
-  // indices of the batch after that are being loaded into registers.
-  constexpr int PER = NB / NT;
-  uint32_t nxt[PER];
-#pragma unroll
-  for (int rr = 0; rr < PER; ++rr) {
-    const uint32_t i = rg.x + tid + rr * NT;
-    if (i < rg.y) cp_async_rec(&s_raw[tid + rr * NT], &P.rec[P.pairs[P.inst_vals[i]]]);
-  }
-  cp_async_commit();
-#pragma unroll
-  for (int rr = 0; rr < PER; ++rr) {
-    const uint32_t i = rg.x + NB + tid + rr * NT;
-    nxt[rr] = i < rg.y ? P.pairs[P.inst_vals[i]] : 0u;
-  }
-
-  for (uint32_t start = rg.x; start < rg.y; start += NB) {
-    if (__syncthreads_and(alive == 0)) {
-      stop_at = start;
-      break;
-    }
-    cp_async_wait_all();  // this thread's raw slots of the batch have landed
-#pragma unroll
-    for (int rr = 0; rr < PER; ++rr) {
-      const int slot = tid + rr * NT;
-      if (start + slot < rg.y)
-        stage_record<DIV>(s_raw[slot], ox_tile, oy_tile, s_A[slot], s_B[slot], s_C[slot], s_D[slot]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int rr = 0; rr < PER; ++rr) {
-      const uint32_t i = start + NB + tid + rr * NT;
-      if (i < rg.y) cp_async_rec(&s_raw[tid + rr * NT], &P.rec[nxt[rr]]);
-    }
-    cp_async_commit();
-#pragma unroll
-    for (int rr = 0; rr < PER; ++rr) {
-      const uint32_t i = start + 2 * NB + tid + rr * NT;
-      nxt[rr] = i < rg.y ? P.pairs[P.inst_vals[i]] : 0u;
-    }
-    const int nb = min(NB, int(rg.y - start));
-    // two records per iteration give the scheduler independent work (8 pixels per thread
-    // would spill)
+// The batch's records (CULL: those of the warp's list), n of them, front to back.  PRE:
+// interleaved columns of the row before the thread's own (compile-time: stepping over them costs
+// its additions alone).
+template <int PX, int PRE, bool CULL, bool COUNT, int DIV>
+__device__ __forceinline__ void composite_batch(const RenderParams &P, Pixels<PX> &S, const float4 *s_A,
+                                                const float4 *s_B, const float4 *s_C, const float4 *s_D,
+                                                const uint8_t *list, int n, int first, float fl_x, float fl_y) {
+  // two records per iteration give the scheduler independent work (8 pixels per thread
+  // would spill)
 #pragma unroll(PX >= 8 ? 1 : 2)
-    for (int j = 0; j < nb && alive; ++j) {
-      const float4 A = s_A[j], B = s_B[j];
-      const float4 Cc = s_C[j];
-      if (COUNT) { n_eval += __popc(alive); ++n_iter; }
-      // with 8 pixels per thread a conservative segment test pays for itself (fewer
-      // pixels per thread are cheaper to test directly); the instrumented variant tests
-      // every pixel, so its image checks the filter
-      if (PX >= 8 && !COUNT && !row_may_hit<PX>(A, B, Cc, s_D[j].w, fl_x, fl_y, step)) continue;
-      float q[PX], r[PX], y0[PX], y1[PX], y2[PX];
-      uint32_t hit = eval_pixels<PX>(A, B, fl_x, fl_y, step, q, r, y0, y1, y2);
-      hit &= alive;
-      if (hit) {
-        const float4 Dd = s_D[j];
+  for (int i = 0; i < n && S.alive; ++i) {
+    const int j = CULL ? list[i] : i;
+    const float4 A = s_A[j], B = s_B[j];
+    const float4 Cc = s_C[j];
+    if (COUNT) { S.n_eval += __popc(S.alive); ++S.n_iter; }
+    // with 8 pixels per thread a conservative segment test pays for itself (fewer
+    // pixels per thread are cheaper to test directly); the instrumented variant tests
+    // every pixel, so its image checks the filters
+    if (PX >= 8 && !COUNT && !row_may_hit<PX>(A, B, Cc, s_D[j].w, fl_x, fl_y, 4.f)) continue;
+    float q[PX], r[PX], y0[PX], y1[PX], y2[PX];
+    uint32_t hit = eval_pixels<PX, PRE>(A, B, fl_x, fl_y, 4.f, q, r, y0, y1, y2);
+    hit &= S.alive;
+    if (hit) {
+      const float4 Dd = s_D[j];
 #pragma unroll
-        for (int k = 0; k < PX; ++k) {
-          if (hit & (1u << k)) {
-            const float al = fminf(P.alpha_max, pixel_opacity<DIV>(Cc, q[k], r[k]));
-            const float w = al * T[k];
-            const float Tn = T[k] - w;
-            if (Tn < P.t_stop) {
-              alive &= ~(1u << k);
-            } else {
-              C0[k] = fmaf(w, Dd.x, C0[k]);
-              C1[k] = fmaf(w, Dd.y, C1[k]);
-              C2[k] = fmaf(w, Dd.z, C2[k]);
-              T[k] = Tn;
-              last[k] = int(start - rg.x) + j + 1;
-              if (COUNT) ++n_comp;
-            }
+      for (int k = 0; k < PX; ++k) {
+        if (hit & (1u << k)) {
+          const float al = fminf(P.alpha_max, pixel_opacity<DIV>(Cc, q[k], r[k]));
+          const float w = al * S.T[k];
+          const float Tn = S.T[k] - w;
+          if (Tn < P.t_stop) {
+            S.alive &= ~(1u << k);
+          } else {
+            S.C0[k] = fmaf(w, Dd.x, S.C0[k]);
+            S.C1[k] = fmaf(w, Dd.y, S.C1[k]);
+            S.C2[k] = fmaf(w, Dd.z, S.C2[k]);
+            S.T[k] = Tn;
+            S.last[k] = first + j + 1;
+            if (COUNT) ++S.n_comp;
           }
         }
       }
     }
   }
+}
+
+template <int NB, int NW>
+struct RasterSmem {
+  float4 A[NB], B[NB], C[NB], D[NB];
+  Rec raw[NB];
+  uint8_t list[NW][NB];  // per warp, the batch's records it keeps 
+  TileItems items;
+};
+
+// Tiles of TW x TH pixels in regions of RW x RH, PX pixels per thread; a warp shades 4 PX columns
+// of eight rows.  CULL: a warp composites only the records whose support can meet one of its
+// pixel centres, listed once per batch.
+template <int TW, int TH, int RW, int RH, int PX, int NBF, bool CULL, bool COUNT, int DIV, typename Smem>
+__device__ __forceinline__ void render_regions(const RenderParams &P, Smem &M) {
+  constexpr int NT = RW * RH / PX;    // threads
+  constexpr int NB = NBF * NT;        // records per batch
+  constexpr int GX = RW / (4 * PX);   // warps side by side
+  constexpr int PX_X = TW / RW, PARTS = PX_X * (TH / RH);
+  static_assert(GX * 4 * PX == RW && RH % 8 == 0 && NB <= 256, "region shape");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const float4 *s_A = M.A, *s_B = M.B, *s_C = M.C, *s_D = M.D;
+  // persistent CTAs: each claims the next item until none is left
+  for (;;) {
+  if (tid == 0) claim_item<PARTS>(P, M.items);
+  __syncthreads();
+  const int tile = M.items.tile, part = M.items.part;
+  if (tile < 0) break;
+  const DevCam &cam = P.cams[M.items.view];
+  const int local = tile - cam.tile_base;
+  const int ty = local / cam.tiles_x, tx = local - ty * cam.tiles_x;
+  const int px0 = tx * TW, py0 = ty * TH;
+  // the warp's first column (in units of four pixels) and row in the tile
+  const int col = (part % PX_X) * (RW / 4) + (warp % GX) * PX, row = (part / PX_X) * RH + (warp / GX) * 8;
+  const int lx = lane & 3, ly = row + (lane >> 2);
+  const int px = px0 + 4 * col + lx, py = py0 + ly;
+  const uint2 rg = P.ranges[tile];
+  const float ox_tile = float(px0) + 0.5f, oy_tile = float(py0) + 0.5f;
+  const float fl_x = float(lx), fl_y = float(ly);
+
+  Pixels<PX> S;
+  S.alive = 0;
+#pragma unroll
+  for (int k = 0; k < PX; ++k) {
+    S.T[k] = 1.f; S.C0[k] = 0.f; S.C1[k] = 0.f; S.C2[k] = 0.f; S.last[k] = 0;
+    if (py < cam.H && px + 4 * k < cam.W) S.alive |= 1u << k;
+  }
+  const uint32_t inside = S.alive;
+  S.n_eval = S.n_comp = S.n_iter = 0;
+  uint32_t stop_at = rg.y;  // first list entry the CTA did not stage
+
+  // Records move through a two-stage pipeline: while a batch is composited, the raw
+  // records of the next batch are in flight to shared memory (cp.async) and the record
+  // indices of the batch after that are being loaded into registers.
+  uint32_t nxt[NBF];
+#pragma unroll
+  for (int rr = 0; rr < NBF; ++rr) {
+    const uint32_t i = rg.x + tid + rr * NT;
+    if (i < rg.y) cp_async_rec(&M.raw[tid + rr * NT], &P.rec[P.pairs[P.inst_vals[i]]]);
+  }
+  cp_async_commit();
+#pragma unroll
+  for (int rr = 0; rr < NBF; ++rr) {
+    const uint32_t i = rg.x + NB + tid + rr * NT;
+    nxt[rr] = i < rg.y ? P.pairs[P.inst_vals[i]] : 0u;
+  }
+
+  for (uint32_t start = rg.x; start < rg.y; start += NB) {
+    if (__syncthreads_and(S.alive == 0)) {
+      stop_at = start;
+      break;
+    }
+    cp_async_wait_all();  // this thread's raw slots of the batch have landed
+#pragma unroll
+    for (int rr = 0; rr < NBF; ++rr) {
+      const int slot = tid + rr * NT;
+      if (start + slot < rg.y)
+        stage_record<DIV>(M.raw[slot], ox_tile, oy_tile, M.A[slot], M.B[slot], M.C[slot], M.D[slot]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int rr = 0; rr < NBF; ++rr) {
+      const uint32_t i = start + NB + tid + rr * NT;
+      if (i < rg.y) cp_async_rec(&M.raw[tid + rr * NT], &P.rec[nxt[rr]]);
+    }
+    cp_async_commit();
+#pragma unroll
+    for (int rr = 0; rr < NBF; ++rr) {
+      const uint32_t i = start + 2 * NB + tid + rr * NT;
+      nxt[rr] = i < rg.y ? P.pairs[P.inst_vals[i]] : 0u;
+    }
+    const int nb = min(NB, int(rg.y - start)), first = int(start - rg.x);
+    int n = nb;
+    uint8_t *list = M.list[CULL ? warp : 0];
+    if (CULL) {
+      n = 0;
+      if (__any_sync(0xffffffffu, S.alive)) {
+#pragma unroll
+        for (int r0 = 0; r0 < NB; r0 += 32) {
+          const int r = r0 + lane;
+          const bool keep = r < nb && box_may_hit(s_A[r], s_B[r], float(4 * col) + (2 * PX - 0.5f),
+                                                  float(row) + 3.5f, 2 * PX - 0.5f, 3.5f);
+          const uint32_t ball = __ballot_sync(0xffffffffu, keep);
+          if (keep) list[n + __popc(ball & ((1u << lane) - 1u))] = uint8_t(r);
+          n += __popc(ball);
+        }
+        __syncwarp();
+      }
+    }
+#define RAYGS_COL(c)                                                                                           \
+  case c:                                                                                                      \
+    if constexpr (c < TW / (4 * PX))                                                                           \
+      composite_batch<PX, (c) * PX, CULL, COUNT, DIV>(P, S, s_A, s_B, s_C, s_D, list, n, first, fl_x, fl_y);         \
+    break;
+    switch (TW == 4 * PX ? 0 : col / PX) {  // (the same for the whole warp)
+      RAYGS_COL(0) RAYGS_COL(1) RAYGS_COL(2) RAYGS_COL(3)
+      RAYGS_COL(4) RAYGS_COL(5) RAYGS_COL(6) RAYGS_COL(7)
+    }
+#undef RAYGS_COL
+  }
   cp_async_wait_all();  // no copy may outlive the block
-  const bool alive_any = COUNT ? __syncthreads_or(alive != 0) : false;
+  const bool alive_any = COUNT ? __syncthreads_or(S.alive != 0) : false;
   if (inside) {
     const long long pix = cam.pix_base + (long long)py * cam.W + px;
 #pragma unroll
     for (int k = 0; k < PX; ++k) {
       if (inside & (1u << k)) {
-        const long long o = pix + k * QX;
-        P.rgb[3 * o] = C0[k];
-        P.rgb[3 * o + 1] = C1[k];
-        P.rgb[3 * o + 2] = C2[k];
-        if (P.Tf) P.Tf[o] = T[k];
-        if (P.ncontrib) P.ncontrib[o] = last[k];
+        const long long o = pix + 4 * k;
+        P.rgb[3 * o] = S.C0[k];
+        P.rgb[3 * o + 1] = S.C1[k];
+        P.rgb[3 * o + 2] = S.C2[k];
+        if (P.Tf) P.Tf[o] = S.T[k];
+        if (P.ncontrib) P.ncontrib[o] = S.last[k];
       }
     }
   }
   if (COUNT) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      n_eval += __shfl_down_sync(0xffffffffu, n_eval, o);
-      n_comp += __shfl_down_sync(0xffffffffu, n_comp, o);
-      n_iter += __shfl_down_sync(0xffffffffu, n_iter, o);
+      S.n_eval += __shfl_down_sync(0xffffffffu, S.n_eval, o);
+      S.n_comp += __shfl_down_sync(0xffffffffu, S.n_comp, o);
+      S.n_iter += __shfl_down_sync(0xffffffffu, S.n_iter, o);
     }
-    if ((tid & 31) == 0) {
-      atomicAdd(&P.eval_counts[0], n_eval);
-      atomicAdd(&P.eval_counts[1], n_comp);
-      atomicAdd(&P.eval_counts[3], n_iter);
+    if (lane == 0) {
+      atomicAdd(&P.eval_counts[0], S.n_eval);
+      atomicAdd(&P.eval_counts[1], S.n_comp);
+      atomicAdd(&P.eval_counts[3], S.n_iter);
     }
     if (tid == 0) {
       atomicAdd(&P.eval_counts[2], (unsigned long long)(stop_at - rg.x));
       if (P.tile_stop) P.tile_stop[tile] = alive_any ? kCulled : stop_at - rg.x;
     }
   }
-  __syncthreads();  // shared state and s_tile are free before the next claim
+  __syncthreads();  // shared state is free before the next claim
   }
 }
 
-// One CTA per resident slot (occupancy of the instantiation x SMs), at most one per tile.
-template <typename K>
-static unsigned persistent_grid(K kernel, int threads, int num_sms, int n_tiles) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm < 1)
-    per_sm = 1;
-  const long long g = (long long)per_sm * (long long)(num_sms > 0 ? num_sms : 1);
-  return unsigned(g < n_tiles ? g : n_tiles);
+// Whole tiles, every record of the list tested by every warp: the variant for many tiles.  Listing
+// each warp's records (CULL) as well made it slower on the stereo batch (4.33 against 4.05 ms):
+// most of a tile's records meet both of its warps.
+template <int TW, int TH, int PX, int NBF, bool COUNT, int DIV>
+__global__ void __launch_bounds__(TW *TH / PX, 16) render_kernel(RenderParams P) {
+  __shared__ RasterSmem<NBF * TW * TH / PX, 1> M;
+  tile_items(P, M.items);
+  render_regions<TW, TH, TW, TH, PX, NBF, false, COUNT, DIV>(P, M);
+  leave_items(P);
+}
+
+// Parts of tiles, for batches of few tiles (launch_render): there the time is that of the tiles
+// with the longest lists, whose records (400 cycles each at four pixels per thread alone, 1,100
+// with the SM full) are composited one after the other.  Two pixels per thread and warps of 8x8
+// pixels that list their records per batch; or, when no more than a fraction of the tiles holds
+// records worth speaking of, one pixel per thread in 8x8 blocks.  A pixel's arithmetic is that of
+// the whole-tile kernel, bit for bit.  720p, 500k primitives: 131 us against 179 in whole tiles
+// (151 with one pixel per thread), 1.5M: 174 against 217 (212); four uneven 640x480 views of 200k:
+// 77 us with one pixel per thread, 117 with two, 191 in whole tiles; 64x64, 1k: 19, 29 and 48.
+template <int TW, int TH, int NBF, int DIV>
+__global__ void __launch_bounds__(64, 18) render_parts_kernel(RenderParams P) {
+  __shared__ RasterSmem<NBF * 64, 2> M;
+  constexpr int RW = TH >= 16 ? 8 : TW >= 16 ? 16 : 8, RH = TH >= 16 ? 16 : 8, PX = RW * RH / 64;
+  tile_items(P, M.items);
+  // tiles with 64 records and more (class 9 is the last of them)
+  static_assert(tile_class_min(9) == 64, "classes");
+  const bool fine = P.class_tiles && M.items.first[10] * uint32_t((TW / 8) * (TH / 8)) <= uint32_t(P.slots);
+  if (PX == 1 || fine) render_regions<TW, TH, 8, 8, 1, NBF, true, false, DIV>(P, M);
+  else render_regions<TW, TH, RW, RH, PX, NBF, true, false, DIV>(P, M);
+  leave_items(P);
+}
+
+template <int TW, int TH, int PX, int NBF, int DIV>
+static cudaError_t run_render(const RenderParams &P, int num_sms, bool count, bool parts, cudaStream_t st) {
+  constexpr int NT = TW * TH / PX;
+  if (count) launch_persistent(render_kernel<TW, TH, PX, NBF, true, DIV>, NT, 1, num_sms, P, st);
+  else if (parts) launch_persistent(render_parts_kernel<TW, TH, NBF, DIV>, 64, (TW / 8) * (TH / 8), num_sms, P, st);
+  else launch_persistent(render_kernel<TW, TH, PX, NBF, false, DIV>, NT, 1, num_sms, P, st);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int batch_records, int num_sms,
                           bool count, cudaStream_t st) {
   if (P.n_tiles <= 0) return cudaSuccess;
   const bool gs = P.qmix == 0.f;  // D_gs records (Sec. 3.1)
-#define RAYGS_RENDER_LAUNCH(TW, TH, PX, NBF, C, D)                                                   \
-  {                                                                                                   \
-    auto k = render_kernel<TW, TH, PX, NBF, C, D>;                                                    \
-    k<<<persistent_grid(k, TW * TH / PX, num_sms, P.n_tiles), TW * TH / PX, 0, st>>>(P);              \
-  }
-#define RAYGS_RENDER_CASE(TW, TH, PX, NBF)                                                             \
-  if (tile_w == TW && tile_h == TH && batch_records == NBF) {                                         \
-    if (gs) {                                                                                         \
-      if (count) RAYGS_RENDER_LAUNCH(TW, TH, PX, NBF, true, 1)                                        \
-      else RAYGS_RENDER_LAUNCH(TW, TH, PX, NBF, false, 1)                                             \
-    } else {                                                                                          \
-      if (count) RAYGS_RENDER_LAUNCH(TW, TH, PX, NBF, true, 0)                                        \
-      else RAYGS_RENDER_LAUNCH(TW, TH, PX, NBF, false, 0)                                             \
-    }                                                                                                 \
-    return cudaGetLastError();                                                                        \
-  }
+  // Parts of tiles up to 2.5 tiles of 16x16 pixels per slot of the whole-tile kernel (16 CTAs per
+  // SM).  500k primitives at 1280x720 (1.5 tiles per slot) 130 against 174 us whole, 1440x810 (1.9)
+  // 141 against 168, 1600x900 (2.3) 154 against 171 (2M primitives: 211 against 210); 1920x1080
+  // (3.4) 194 against 187, 2560x1440 (5.9) 292 against 259.
+  const bool parts = 2 * int64_t(P.n_tiles) * tile_w * tile_h <= 5 * int64_t(num_sms) * 16 * 256;
+#define RAYGS_RENDER_CASE(TW, TH, PX, NBF)                                                       \
+  if (tile_w == TW && tile_h == TH && batch_records == NBF)                                     \
+    return gs ? run_render<TW, TH, PX, NBF, 1>(P, num_sms, count, parts, st)                    \
+              : run_render<TW, TH, PX, NBF, 0>(P, num_sms, count, parts, st);
   RAYGS_RENDER_CASE(16, 16, 4, 1)
   RAYGS_RENDER_CASE(16, 8, 4, 1)
   RAYGS_RENDER_CASE(32, 16, 8, 1)
@@ -223,7 +298,6 @@ cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int bat
   RAYGS_RENDER_CASE(32, 16, 8, 2)
   RAYGS_RENDER_CASE(8, 8, 2, 2)
 #undef RAYGS_RENDER_CASE
-#undef RAYGS_RENDER_LAUNCH
   return cudaErrorInvalidValue;
 }
 

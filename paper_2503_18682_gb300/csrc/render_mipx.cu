@@ -186,10 +186,9 @@ __global__ void __launch_bounds__(TW *TH / PX, 8) render_mipx_kernel(RenderParam
   }
 }
 
-cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int64_t n_tiles, bool count,
+cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int num_sms, bool count,
                                cudaStream_t st) {
-  if (n_tiles == 0) return cudaSuccess;
-  const unsigned grid = unsigned(n_tiles);
+  const unsigned grid = unsigned(P.n_tiles);
 #define RAYGS_MIPX_CASE(TW, TH, PX)                                                        \
   if (tile_w == TW && tile_h == TH) {                                                      \
     if (count) render_mipx_kernel<TW, TH, PX, true><<<grid, TW * TH / PX, 0, st>>>(P);     \
