@@ -16,30 +16,34 @@
 
 namespace raygs {
 
-template <int TW, int TH, int PX, bool COUNT>
-__global__ void __launch_bounds__(TW *TH / PX, 8) render_mipx_kernel(RenderParams P) {
-  constexpr int NT = TW * TH / PX;  // threads; one record per thread and batch
-  constexpr int QX = TW / PX;       // threads per tile row
+// Tiles of TW x TH pixels in regions of RW x RH, PX pixels per thread (the region shapes and the
+// claiming of items are those of render.cu).
+template <int TW, int TH, int RW, int RH, int PX, bool COUNT>
+__global__ void __launch_bounds__(RW *RH / PX, PX >= 4 ? 8 : PX == 2 ? 10 : 14) render_mipx_kernel(RenderParams P) {
+  constexpr int NT = RW * RH / PX;  // threads; one record per thread and batch
+  constexpr int GX = RW / (4 * PX), PX_X = TW / RW, PARTS = PX_X * (TH / RH);
+  static_assert(GX * 4 * PX == RW && RH % 8 == 0, "region shape");
   __shared__ float4 s_S[7][NT];
   __shared__ Rec s_raw[2][NT];
-  __shared__ int s_view;
-  const int tile = blockIdx.x;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    int v = 0;
-    while (v + 1 < P.n_views && P.cams[v + 1].tile_base <= tile) ++v;
-    s_view = v;
-  }
+  __shared__ TileItems s_items;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  tile_items(P, s_items);
+  for (;;) {
+  if (tid == 0) claim_item<PARTS>(P, s_items);
   __syncthreads();
-  const DevCam &cam = P.cams[s_view];
+  const int tile = s_items.tile, part = s_items.part;
+  if (tile < 0) break;
+  const DevCam &cam = P.cams[s_items.view];
   const int local = tile - cam.tile_base;
   const int ty = local / cam.tiles_x, tx = local - ty * cam.tiles_x;
   const int px0 = tx * TW, py0 = ty * TH;
-  const int lx = tid % QX, ly = tid / QX;
-  const int px = px0 + lx, py = py0 + ly;
+  const int col = (part % PX_X) * (RW / 4) + (warp % GX) * PX, row = (part / PX_X) * RH + (warp / GX) * 8;
+  const int lx = lane & 3, ly = row + (lane >> 2);
+  const int px = px0 + 4 * col + lx, py = py0 + ly;
+  constexpr int QX = 4;  // a row's pixels lie in four interleaved columns
   const uint2 rg = P.ranges[tile];
   const float ox_tile = float(px0) + 0.5f, oy_tile = float(py0) + 0.5f;
-  const float fl_x = float(lx), fl_y = float(ly), step = float(QX);
+  const float fl_x = float(lx), fl_y = float(ly), step = float(QX), skip = float(col);
   const float c2h = 0.5f * kLog2e;
 
   float T[PX], C0[PX], C1[PX], C2[PX], ixn[PX];
@@ -112,7 +116,7 @@ __global__ void __launch_bounds__(TW *TH / PX, 8) render_mipx_kernel(RenderParam
       uint32_t hit = 0;
 #pragma unroll
       for (int k = 0; k < PX; ++k) {
-        const float dx = dx0 + float(k) * step;
+        const float dx = dx0 + (skip + float(k)) * step;
         const float e0 = fmaf(S0.z, dx, e0r), e1 = fmaf(S1.x, dx, e1r), e2 = fmaf(S1.z, dx, e2r);
         const float y0 = fmaf(S2.x, dx, y0r), y1 = fmaf(S2.z, dx, y1r), y2 = fmaf(S3.x, dx, y2r);
         const float my0 = S4.y * y0, my1 = S4.z * y1, my2 = S4.w * y2;
@@ -184,22 +188,38 @@ __global__ void __launch_bounds__(TW *TH / PX, 8) render_mipx_kernel(RenderParam
       atomicAdd(&P.eval_counts[1], n_comp);
     }
   }
+  __syncthreads();  // shared state is free before the next claim
+  }
+  leave_items(P);
+}
+
+// Two pixels per thread: at four the kernel needs 117 registers (8 CTAs of 64 threads per SM) and
+// was the slower one at every size (500k primitives: 458 against 350-373 us at 1280x720, 609
+// against 521 at 1920x1080, 901 against 776 at 2560x1440; 1M at 3840x2160 2.28 against 1.96 ms).
+// By the tiles (of 16x16 pixels) per slot of 16 CTAs per SM, as in render.cu: up to 0.75, 8x8 blocks with
+// one pixel per thread (640x360, 200k primitives, 0.4: 285 us, two pixels 358 to 428; 160x120, 20k: 121
+// against 172), where the longest list sets the time; up to 2.5, 8x8 blocks with two (720p, 1.5: 350
+// against 373 in 8x16; with 1.5M primitives 504 against 517); else 8x16 regions (1080p, 3.4: 521
+// against 529; 4K, 13: 1.96 against 2.02 ms).
+template <int TW, int TH, int PX>
+static cudaError_t run_mipx(const RenderParams &P, int num_sms, bool count, cudaStream_t st) {
+  constexpr int RW = TH >= 16 ? 8 : TW >= 16 ? 16 : 8, RH = TH >= 16 ? 16 : 8;
+  constexpr int BLOCKS = (TW / 8) * (TH / 8);
+  const int64_t area = int64_t(P.n_tiles) * TW * TH, slots = int64_t(num_sms) * 16 * 256;
+  if (count) launch_persistent(render_mipx_kernel<TW, TH, TW, TH, PX, true>, TW * TH / PX, 1, num_sms, P, st);
+  else if (4 * area <= 3 * slots) launch_persistent(render_mipx_kernel<TW, TH, 8, 8, 1, false>, 64, BLOCKS, num_sms, P, st);
+  else if (2 * area <= 5 * slots) launch_persistent(render_mipx_kernel<TW, TH, 8, 8, 2, false>, 32, BLOCKS, num_sms, P, st);
+  else launch_persistent(render_mipx_kernel<TW, TH, RW, RH, 2, false>, RW * RH / 2, BLOCKS * 64 / (RW * RH), num_sms, P, st);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int num_sms, bool count,
                                cudaStream_t st) {
-  const unsigned grid = unsigned(P.n_tiles);
-#define RAYGS_MIPX_CASE(TW, TH, PX)                                                        \
-  if (tile_w == TW && tile_h == TH) {                                                      \
-    if (count) render_mipx_kernel<TW, TH, PX, true><<<grid, TW * TH / PX, 0, st>>>(P);     \
-    else render_mipx_kernel<TW, TH, PX, false><<<grid, TW * TH / PX, 0, st>>>(P);          \
-    return cudaGetLastError();                                                             \
-  }
-  RAYGS_MIPX_CASE(16, 16, 4)
-  RAYGS_MIPX_CASE(16, 8, 4)
-  RAYGS_MIPX_CASE(32, 16, 8)
-  RAYGS_MIPX_CASE(8, 8, 2)
-#undef RAYGS_MIPX_CASE
+  if (P.n_tiles <= 0) return cudaSuccess;
+  if (tile_w == 16 && tile_h == 16) return run_mipx<16, 16, 4>(P, num_sms, count, st);
+  if (tile_w == 16 && tile_h == 8) return run_mipx<16, 8, 4>(P, num_sms, count, st);
+  if (tile_w == 32 && tile_h == 16) return run_mipx<32, 16, 8>(P, num_sms, count, st);
+  if (tile_w == 8 && tile_h == 8) return run_mipx<8, 8, 2>(P, num_sms, count, st);
   return cudaErrorInvalidValue;
 }
 

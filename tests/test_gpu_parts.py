@@ -33,3 +33,14 @@ def test_parts_equal_whole_tiles(tile, batch_records, divergence):
     scene["log_scales"][:2000, 1] -= 5.0
     view = scenes.make_camera(633, 478, 420.0, 430.0)
     _same(scene, view, [view] * 8, **cfg)
+
+
+@pytest.mark.parametrize("tile", [(16, 16), (16, 8), (32, 16), (8, 8)])
+def test_exact_antialiasing_parts(tile):
+    """The exact anti-aliasing's region shapes (8x8 blocks with one or two pixels per thread, larger
+    regions with two) give the same bits."""
+    cfg = dict(tile_w=tile[0], tile_h=tile[1])
+    scene = scenes.uniform_scene(2500, seed=93)
+    small = scenes.make_camera(171, 149, 150.0, 140.0, mip="exact")
+    _same(scene, small, [small] * 30, **cfg)            # alone one pixel; 3,300 tiles: two in blocks
+    _same(scene, small, [small] * 64, **cfg)            # 7,040 tiles: larger regions
