@@ -115,6 +115,8 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.deg = L.s1k[0];  // the FP64 lists of the vertex stage and of the backward: free then
   L.degc = take(4);
   L.partials = backward ? take(4 * kGradW * C + 16) : 0;
+  L.ptouch = backward ? take(C + 16) : 0;
+  L.pgtouch = backward ? take(VN + 16) : 0;
   L.pg = backward ? take(4 * kGradW * VN + 16) : 0;
   L.total = o;
   return L;
@@ -337,8 +339,16 @@ cudaError_t run_backward(const Work &w, const raygs_scene &scene, const float *T
   B.dL_drgb = dL_drgb;
   B.dL_dT = dL_dT;
   B.partials = w.at<float>(w.L.partials);
-  cudaError_t e = launch_render_backward(B, w.cfg.tile_w, w.cfg.tile_h, w.tiles, st);
+  B.touched = w.at<uint8_t>(w.L.ptouch);
+  B.tile_counter = w.at<unsigned int>(w.L.tilectr);
+  B.n_tiles = int(w.tiles);
+  B.counters = w.at<Counters>(w.L.counters);
+  B.class_tiles = w.L.tclass ? w.at<uint32_t>(w.L.tclass) : nullptr;
+  cudaError_t e = cudaMemsetAsync(B.touched, 0, size_t(w.cap), st);
   if (e != cudaSuccess) return e;
+  uint8_t *pair_touched = w.at<uint8_t>(w.L.pgtouch);
+  if ((e = cudaMemsetAsync(pair_touched, 0, size_t(w.n_views) * size_t(w.n), st)) != cudaSuccess) return e;
+  if ((e = launch_render_backward(B, w.cfg.tile_w, w.cfg.tile_h, w.num_sms, st)) != cudaSuccess) return e;
   PairGradParams Q{};
   Q.pairs = B.pairs;
   Q.pair_e = w.at<uint4>(w.L.paire);
@@ -346,7 +356,9 @@ cudaError_t run_backward(const Work &w, const raygs_scene &scene, const float *T
   Q.cap = B.cap;
   Q.counters = w.at<Counters>(w.L.counters);
   Q.partials = B.partials;
+  Q.touched = B.touched;
   Q.pg = w.at<float>(w.L.pg);
+  Q.pair_touched = pair_touched;
   if ((e = launch_pair_grads(Q, w.G, st)) != cudaSuccess) return e;
   ParamGradParams R{};
   R.means = scene.means;
@@ -364,7 +376,7 @@ cudaError_t run_backward(const Work &w, const raygs_scene &scene, const float *T
   R.p_min = w.cfg.p_min;
   R.degenerate_ratio = w.cfg.degenerate_ratio;
   R.fp64_degenerate = w.cfg.fp64_degenerate;
-  R.depth_key = w.at<uint32_t>(w.L.depth);
+  R.pair_touched = pair_touched;
   R.pg = Q.pg;
   R.d_means = grads.d_means;
   R.d_log_scales = grads.d_log_scales;

@@ -324,6 +324,11 @@ struct BackParams {
   const float *dL_drgb;
   const float *dL_dT;   // nullable
   float *partials;      // [capacity][kGradW] by partial-sum slot
+  uint8_t *touched;     // [capacity] slots that hold a partial sum (cleared first; the others are zero)
+  unsigned int *tile_counter;  // as in RenderParams
+  const Counters *counters;
+  const uint32_t *class_tiles;
+  int n_tiles, slots;
 };
 
 struct PairGradParams {
@@ -333,7 +338,9 @@ struct PairGradParams {
   uint32_t cap;
   const Counters *counters;
   const float *partials;
-  float *pg;            // [V*N][kGradW] by pair id
+  const uint8_t *touched;
+  float *pg;            // [V*N][kGradW] by pair id, of the pairs with a gradient
+  uint8_t *pair_touched;  // [V*N] pairs with a gradient (cleared first)
 };
 
 struct ParamGradParams {
@@ -347,7 +354,7 @@ struct ParamGradParams {
   const DevCam *cams;
   float p_min, degenerate_ratio;
   int fp64_degenerate;
-  const uint32_t *depth_key;
+  const uint8_t *pair_touched;  // [V*N] pairs with a gradient
   const float *pg;
   float *d_means, *d_log_scales, *d_quats, *d_logits, *d_sh;
   int num_sms;
@@ -371,7 +378,7 @@ cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int bat
                           bool count, cudaStream_t st);
 cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int num_sms, bool count,
                                cudaStream_t st);
-cudaError_t launch_render_backward(const BackParams &P, int tile_w, int tile_h, int64_t n_tiles, cudaStream_t st);
+cudaError_t launch_render_backward(const BackParams &P, int tile_w, int tile_h, int num_sms, cudaStream_t st);
 cudaError_t launch_pair_grads(const PairGradParams &P, int G, cudaStream_t st);
 cudaError_t launch_param_grads(const ParamGradParams &P, cudaStream_t st);
 cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo, float *T_lo, int w_lo, int h_lo,
@@ -381,7 +388,7 @@ cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo
 // Byte offsets of every buffer inside one caller-owned (or library-static) workspace.
 struct Layout {
   size_t tilectr, tclass, cams, spanl, spans, vpos, counters, evals, tstop, depth, rect, rinfo, ell, rec, recx, s1k[2], s1v[2], cnt1, trcnt, rows,
-      re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, pg, total;
+      re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, ptouch, pg, pgtouch, total;
 };
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
