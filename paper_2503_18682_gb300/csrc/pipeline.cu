@@ -115,6 +115,8 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.deg = L.s1k[0];  // the FP64 lists of the vertex stage and of the backward: free then
   L.degc = take(4);
   L.partials = backward ? take(4 * kGradW * C + 16) : 0;
+  L.bclass = backward ? take(4 * size_t(kTileClasses) * size_t(tiles) + 16) : 0;
+  L.bplan = backward ? take(sizeof(ReplayPlan)) : 0;
   L.ptouch = backward ? take(C + 16) : 0;
   L.pgtouch = backward ? take(VN + 16) : 0;
   L.pg = backward ? take(4 * kGradW * VN + 16) : 0;
@@ -315,8 +317,8 @@ cudaError_t run_render(const Work &w, float *rgb, float *T_final, int32_t *n_con
   if (w.tiles == 0) return cudaSuccess;
   P.tile_counter = w.at<unsigned int>(w.L.tilectr);
   P.n_tiles = int(w.tiles);
-  P.counters = w.at<Counters>(w.L.counters);
   P.class_tiles = w.L.tclass ? w.at<uint32_t>(w.L.tclass) : nullptr;
+  P.class_count = w.at<Counters>(w.L.counters)->tile_class;
   if (P.recx) return launch_render_mipx(P, w.cfg.tile_w, w.cfg.tile_h, w.num_sms, count, st);
   return launch_render(P, w.cfg.tile_w, w.cfg.tile_h, w.cfg.batch_records, w.num_sms, count, st);
 }
@@ -342,13 +344,15 @@ cudaError_t run_backward(const Work &w, const raygs_scene &scene, const float *T
   B.touched = w.at<uint8_t>(w.L.ptouch);
   B.tile_counter = w.at<unsigned int>(w.L.tilectr);
   B.n_tiles = int(w.tiles);
-  B.counters = w.at<Counters>(w.L.counters);
-  B.class_tiles = w.L.tclass ? w.at<uint32_t>(w.L.tclass) : nullptr;
-  cudaError_t e = cudaMemsetAsync(B.touched, 0, size_t(w.cap), st);
-  if (e != cudaSuccess) return e;
+  B.plan = w.at<ReplayPlan>(w.L.bplan);
+  B.class_tiles = w.at<uint32_t>(w.L.bclass);
+  B.class_count = B.plan->tile_class;
+  B.num_sms = w.num_sms > 0 ? w.num_sms : 1;
   uint8_t *pair_touched = w.at<uint8_t>(w.L.pgtouch);
-  if ((e = cudaMemsetAsync(pair_touched, 0, size_t(w.n_views) * size_t(w.n), st)) != cudaSuccess) return e;
-  if ((e = launch_render_backward(B, w.cfg.tile_w, w.cfg.tile_h, w.num_sms, st)) != cudaSuccess) return e;
+  // the plan, touched and pair_touched lie behind one another: one clear
+  cudaError_t e = cudaMemsetAsync(B.plan, 0, w.L.pgtouch - w.L.bplan + size_t(w.n_views) * size_t(w.n), st);
+  if (e != cudaSuccess) return e;
+  if ((e = launch_render_backward(B, w.cfg.tile_w, w.cfg.tile_h, st)) != cudaSuccess) return e;
   PairGradParams Q{};
   Q.pairs = B.pairs;
   Q.pair_e = w.at<uint4>(w.L.paire);

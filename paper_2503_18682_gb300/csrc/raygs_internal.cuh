@@ -291,8 +291,8 @@ struct RenderParams {
   unsigned int *tile_counter;  // [0] next unclaimed item of the persistent rasteriser, [1] CTAs that
                                // have left it; both 0 between launches (the last CTA clears them)
   int n_tiles;
-  const Counters *counters;
   const uint32_t *class_tiles;  // tiles by class (nullable: tile order)
+  const uint32_t *class_count;
   int slots;                    // CTAs resident at a time (set at the launch)
   const Rec *recx;  // exact anti-aliasing: second half of each record (then rec holds the first)
   float p_min;
@@ -308,6 +308,12 @@ struct RenderParams {
 
 constexpr int kMaxTilesX = 4096;  // tiles in one tile row (32768-pixel views at 8-pixel tiles)
 constexpr int kGradW = 13;  // per-instance / per-pair gradient partials (see backward.cu)
+
+// What a backward pass has to replay: the lists up to the last composited instance.
+struct ReplayPlan {
+  uint32_t longest, sum;  // over the tiles
+  uint32_t tile_class[kTileClasses];  // tiles of each class, without those that have nothing to replay
+};
 
 struct BackParams {
   const DevCam *cams;
@@ -326,9 +332,10 @@ struct BackParams {
   float *partials;      // [capacity][kGradW] by partial-sum slot
   uint8_t *touched;     // [capacity] slots that hold a partial sum (cleared first; the others are zero)
   unsigned int *tile_counter;  // as in RenderParams
-  const Counters *counters;
-  const uint32_t *class_tiles;
-  int n_tiles, slots;
+  ReplayPlan *plan;            // cleared first
+  uint32_t *class_tiles;       // nullable, the tiles of each class of the plan
+  const uint32_t *class_count;
+  int n_tiles, slots, num_sms;
 };
 
 struct PairGradParams {
@@ -378,7 +385,7 @@ cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int bat
                           bool count, cudaStream_t st);
 cudaError_t launch_render_mipx(const RenderParams &P, int tile_w, int tile_h, int num_sms, bool count,
                                cudaStream_t st);
-cudaError_t launch_render_backward(const BackParams &P, int tile_w, int tile_h, int num_sms, cudaStream_t st);
+cudaError_t launch_render_backward(const BackParams &P, int tile_w, int tile_h, cudaStream_t st);
 cudaError_t launch_pair_grads(const PairGradParams &P, int G, cudaStream_t st);
 cudaError_t launch_param_grads(const ParamGradParams &P, cudaStream_t st);
 cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo, float *T_lo, int w_lo, int h_lo,
@@ -388,7 +395,7 @@ cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo
 // Byte offsets of every buffer inside one caller-owned (or library-static) workspace.
 struct Layout {
   size_t tilectr, tclass, cams, spanl, spans, vpos, counters, evals, tstop, depth, rect, rinfo, ell, rec, recx, s1k[2], s1v[2], cnt1, trcnt, rows,
-      re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, ptouch, pg, pgtouch, total;
+      re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, bclass, bplan, ptouch, pg, pgtouch, total;
 };
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
