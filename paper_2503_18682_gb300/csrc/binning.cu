@@ -46,6 +46,7 @@ __device__ __forceinline__ uint32_t pass_count(const SortPass &p) {
 // in order) and adds each run once to its warp's shared histogram.
 template <int BITS, bool FILTER>
 __global__ void __launch_bounds__(kSortThreads) sort_upsweep(SortPass p) {
+  await_previous();
   constexpr int R = 1 << BITS;
   constexpr int KPT = 16;  // keys per thread per step
   __shared__ uint32_t h[kSortWarps][R];
@@ -99,6 +100,7 @@ enum SortMode { kSortPlain = 0, kSortFirst = 1, kSortLast = 2, kSortSplit = 3 };
 
 template <int BITS, int MODE>
 __global__ void __launch_bounds__(kSortThreads, 4) sort_downsweep(SortPass p) {
+  await_previous();
   constexpr int R = 1 << BITS;
   __shared__ uint32_t s_keys[kSortTile];
   __shared__ uint32_t s_vals[kSortTile];
@@ -263,6 +265,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) sort_downsweep(SortPass p) {
 constexpr int kSortMaxGrid = 1024;
 
 __global__ void __launch_bounds__(256) hist_scan_kernel(uint32_t *hist, int G, uint32_t *digit_total) {
+  await_previous();
   __shared__ uint32_t ws[33];
   constexpr int PER = kSortMaxGrid / 256;
   uint32_t *row = hist + size_t(blockIdx.x) * G;
@@ -291,9 +294,9 @@ __global__ void __launch_bounds__(256) hist_scan_kernel(uint32_t *hist, int G, u
 // costs more than the launch.
 template <int BITS, int MODE>
 static cudaError_t sort_pass(const SortPass &p, cudaStream_t st) {
-  sort_upsweep<BITS, MODE == kSortFirst><<<p.G, kSortThreads, 0, st>>>(p);
-  if (p.G > kSortNoScan) hist_scan_kernel<<<1 << BITS, 256, 0, st>>>(p.hist, p.G, p.digit_total);
-  sort_downsweep<BITS, MODE><<<p.G, kSortThreads, 0, st>>>(p);
+  launch(sort_upsweep<BITS, MODE == kSortFirst>, p.G, kSortThreads, 0, st, p);
+  if (p.G > kSortNoScan) launch(hist_scan_kernel, 1 << BITS, 256, 0, st, p.hist, p.G, p.digit_total);
+  launch(sort_downsweep<BITS, MODE>, p.G, kSortThreads, 0, st, p);
   return cudaGetLastError();
 }
 

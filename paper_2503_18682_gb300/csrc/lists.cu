@@ -86,6 +86,7 @@ __device__ void scan_trow_instances(const ListParams &P) {
 // Instances per tile column of one chunk: each row covers the tile columns
 // [txa, txa + len); a difference array over the columns and its prefix sum count them.
 __global__ void __launch_bounds__(256) list_count_kernel(ListParams P) {
+  await_previous();
   extern __shared__ uint32_t s_diff[];  // [max_tiles_x + 1]
   __shared__ uint32_t s_ws[33];
   __shared__ bool s_last;
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(256) list_count_kernel(ListParams P) {
 // rows of the next step are loaded during this one.
 template <int NT, int KR>
 __global__ void __launch_bounds__(NT) list_kernel(ListParams P) {
+  await_previous();
   constexpr int VW = NT / 32 * KR;  // row groups per step
   extern __shared__ uint32_t s_mem[];
   int grow, chunk_c;
@@ -300,14 +302,14 @@ uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sm
 cudaError_t launch_lists(const ListParams &P, int num_sms, cudaStream_t st) {
   if (P.trows == 0) return cudaSuccess;
   const unsigned cg = unsigned(std::min<uint64_t>(P.max_chunks, uint64_t(num_sms) * 8));
-  list_count_kernel<<<cg, 256, sizeof(uint32_t) * size_t(P.max_tiles_x + 1), st>>>(P);
+  launch(list_count_kernel, cg, 256, sizeof(uint32_t) * size_t(P.max_tiles_x + 1), st, P);
   constexpr size_t kBudget = 200 * 1024;
   auto run = [&](auto kernel, int nt, size_t smem) -> cudaError_t {
     if (smem > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
       if (e != cudaSuccess) return e;
     }
-    kernel<<<P.max_chunks, nt, smem, st>>>(P);
+    launch(kernel, P.max_chunks, nt, smem, st, P);
     return cudaGetLastError();
   };
   const int mtx = P.max_tiles_x;

@@ -82,6 +82,7 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.cams = take(sizeof(DevCam) * size_t(n_views));
   L.counters = take(sizeof(Counters) + 16);  // and the rasteriser's tile counter
   L.tilectr = L.counters + sizeof(Counters);
+  L.degc = L.tilectr + 8;  // cleared with the counters
   L.evals = take(4 * sizeof(unsigned long long));
   L.depth = take(4 * VN);
   L.rect = take(8 * VN);
@@ -113,7 +114,6 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.tclass = tile_order ? take(4 * size_t(kTileClasses) * size_t(tiles) + 16) : 0;
   L.tstop = take(4 * size_t(tiles) + 16);
   L.deg = L.s1k[0];  // the FP64 lists of the vertex stage and of the backward: free then
-  L.degc = take(4);
   L.partials = backward ? take(4 * kGradW * C + 16) : 0;
   L.bclass = backward ? take(4 * size_t(kTileClasses) * size_t(tiles) + 16) : 0;
   L.bplan = backward ? take(sizeof(ReplayPlan)) : 0;
@@ -389,8 +389,7 @@ cudaError_t run_backward(const Work &w, const raygs_scene &scene, const float *T
   R.d_sh = grads.d_sh;
   R.num_sms = w.num_sms;
   R.fp64_list = w.at<uint32_t>(w.L.deg);
-  R.fp64_count = w.at<uint32_t>(w.L.degc);
-  if ((e = cudaMemsetAsync(R.fp64_count, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
+  R.fp64_count = &B.plan->fp64_count;
   return launch_param_grads(R, st);
 }
 

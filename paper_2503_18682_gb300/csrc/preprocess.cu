@@ -552,6 +552,7 @@ __device__ __forceinline__ int stage_for(const T mu[3], const T Rp[9], const T s
 
 template <int DEG, int MODE>
 __global__ void __launch_bounds__(kPrepThreads) preprocess_kernel(PrepParams P) {
+  await_previous();
   constexpr int K3 = 3 * (DEG + 1) * (DEG + 1);
   // padded SH row: whole 16-byte slots, an odd number of them
   constexpr int K4 = (K3 + 3) / 4;
@@ -733,6 +734,7 @@ __global__ void __launch_bounds__(kPrepThreads) preprocess_kernel(PrepParams P) 
 // device-side list.
 template <int DEG, int MODE>
 __global__ void __launch_bounds__(128) preprocess_fp64_kernel(PrepParams P) {
+  await_previous();
   constexpr int K = (DEG + 1) * (DEG + 1);
   const uint32_t count = *P.deg_count;
   for (uint32_t li = blockIdx.x * blockDim.x + threadIdx.x; li < count; li += gridDim.x * blockDim.x) {
@@ -776,9 +778,8 @@ cudaError_t launch_preprocess(const PrepParams &P, int num_sms, cudaStream_t st)
   if (P.n == 0) return cudaSuccess;
   int blocks = (P.n + kPrepThreads - 1) / kPrepThreads;
   size_t dyn = sizeof(DevCam) * P.n_views;
-  cudaMemsetAsync(P.deg_count, 0, sizeof(uint32_t), st);
   const int mode = P.divergence == 1 ? kStageGS : P.recx ? kStageExact : kStageRay;
-#define RAYGS_PREP(D, M) preprocess_kernel<D, M><<<blocks, kPrepThreads, dyn, st>>>(P)
+#define RAYGS_PREP(D, M) launch(preprocess_kernel<D, M>, blocks, kPrepThreads, dyn, st, P)
 #define RAYGS_PREP_MODES(D)                 \
   if (mode == kStageGS) RAYGS_PREP(D, 1);         \
   else if (mode == kStageExact) RAYGS_PREP(D, 2); \
@@ -795,7 +796,7 @@ cudaError_t launch_preprocess(const PrepParams &P, int num_sms, cudaStream_t st)
   if (e != cudaSuccess) return e;
   {  // the listed pairs: near-degenerate ones and undecided skip decisions
     int gb = num_sms * 4;
-#define RAYGS_FP64(D, M) preprocess_fp64_kernel<D, M><<<gb, 128, 0, st>>>(P)
+#define RAYGS_FP64(D, M) launch(preprocess_fp64_kernel<D, M>, gb, 128, 0, st, P)
 #define RAYGS_FP64_MODES(D)                 \
   if (mode == kStageGS) RAYGS_FP64(D, 1);         \
   else if (mode == kStageExact) RAYGS_FP64(D, 2); \

@@ -240,6 +240,7 @@ __device__ __forceinline__ void render_regions(const RenderParams &P, Smem &M) {
 // most of a tile's records meet both of its warps.
 template <int TW, int TH, int PX, int NBF, bool COUNT, int DIV>
 __global__ void __launch_bounds__(TW *TH / PX, 16) render_kernel(RenderParams P) {
+  await_previous();
   __shared__ RasterSmem<NBF * TW * TH / PX, 1> M;
   tile_items(P, M.items);
   render_regions<TW, TH, TW, TH, PX, NBF, false, COUNT, DIV>(P, M);
@@ -256,6 +257,7 @@ __global__ void __launch_bounds__(TW *TH / PX, 16) render_kernel(RenderParams P)
 // 77 us with one pixel per thread, 117 with two, 191 in whole tiles; 64x64, 1k: 19, 29 and 48.
 template <int TW, int TH, int NBF, int DIV>
 __global__ void __launch_bounds__(64, 18) render_parts_kernel(RenderParams P) {
+  await_previous();
   __shared__ RasterSmem<NBF * 64, 2> M;
   constexpr int RW = TH >= 16 ? 8 : TW >= 16 ? 16 : 8, RH = TH >= 16 ? 16 : 8, PX = RW * RH / 64;
   tile_items(P, M.items);

@@ -20,6 +20,7 @@ namespace raygs {
 // claiming of items are those of render.cu).
 template <int TW, int TH, int RW, int RH, int PX, bool COUNT>
 __global__ void __launch_bounds__(RW *RH / PX, PX >= 4 ? 8 : PX == 2 ? 10 : 14) render_mipx_kernel(RenderParams P) {
+  await_previous();
   constexpr int NT = RW * RH / PX;  // threads; one record per thread and batch
   constexpr int GX = RW / (4 * PX), PX_X = TW / RW, PARTS = PX_X * (TH / RH);
   static_assert(GX * 4 * PX == RW && RH % 8 == 0, "region shape");

@@ -9,6 +9,7 @@ namespace raygs {
 __global__ void __launch_bounds__(256) resolve_kernel(const float *rgb_hi, const float *T_hi, float *rgb_lo,
                                                       float *T_lo, int w_lo, int h_lo, int factor,
                                                       long long base_hi, long long base_lo) {
+  await_previous();
   const long long n = (long long)w_lo * h_lo;
   const int w_hi = w_lo * factor;
   const float inv = 1.f / float(factor * factor);
@@ -38,8 +39,8 @@ cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo
   const long long n = (long long)w_lo * h_lo;
   if (n == 0) return cudaSuccess;
   const long long blocks = (n + 255) / 256;
-  resolve_kernel<<<unsigned(blocks < 65535 ? blocks : 65535), 256, 0, st>>>(rgb_hi, T_hi, rgb_lo, T_lo, w_lo, h_lo,
-                                                                           factor, base_hi, base_lo);
+  launch(resolve_kernel, unsigned(blocks < 65535 ? blocks : 65535), 256, 0, st, rgb_hi, T_hi, rgb_lo, T_lo, w_lo, h_lo,
+         factor, base_hi, base_lo);
   return cudaGetLastError();
 }
 

@@ -335,6 +335,7 @@ __device__ __forceinline__ void scan_rows(const PlaceParams &P) {
 // shared memory, two atomics per pair.
 template <int J>
 __global__ void __launch_bounds__(32 * kPlaceWarps) pair_count_kernel(PlaceParams P, int nj_dyn) {
+  await_previous();
   constexpr int NW = kPlaceWarps;
   extern __shared__ __align__(16) unsigned char s_count[];
   __shared__ ViewTab T;
@@ -371,6 +372,7 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) pair_count_kernel(PlaceParam
 // One CTA per tile row: exclusive scan of its chunks' counts in place, and their total; then
 // the rows left to be scanned.
 __global__ void __launch_bounds__(256) row_base_kernel(PlaceParams P) {
+  await_previous();
   __shared__ ViewTab T;
   __shared__ uint32_t ws[33];
   build_view_tab(P, T);
@@ -435,6 +437,7 @@ __device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long lo
 // capacity: every slot below it belongs to exactly one row), the row total, the capacity
 // check, the chunks of the list pass, and its instance totals cleared.
 __global__ void __launch_bounds__(1024) trow_plan_kernel(PlaceParams P) {
+  await_previous();
   __shared__ unsigned long long ws[33];
   const int per = (P.trows + 1023) / 1024;
   const int b = min(P.trows, int(threadIdx.x) * per), e = min(P.trows, b + per);
@@ -506,6 +509,7 @@ static size_t place_smem(int nj) {
 
 template <int J, bool BWD>
 __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, int nj_dyn) {
+  await_previous();
   constexpr int NW = kPlaceWarps;
   extern __shared__ __align__(16) unsigned char s_place[];
   __shared__ ViewTab T;
@@ -666,10 +670,10 @@ static cudaError_t run_place(const PlaceParams &P, int nj, int num_sms, uint64_t
     e = cudaFuncSetAttribute(pair_count_kernel<J>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(csmem));
   if (e != cudaSuccess) return e;
   const uint64_t ctas = (max_chunks + NW - 1) / NW;
-  pair_count_kernel<J><<<unsigned(std::min<uint64_t>(ctas, uint64_t(num_sms) * 8)), 32 * NW, csmem, st>>>(P, nj);
-  row_base_kernel<<<P.trows, 256, 0, st>>>(P);
-  trow_plan_kernel<<<1, 1024, 0, st>>>(P);
-  place_kernel<J, BWD><<<unsigned(std::min<uint64_t>(ctas, uint64_t(num_sms) * 16)), 32 * NW, smem, st>>>(P, nj);
+  launch(pair_count_kernel<J>, unsigned(std::min<uint64_t>(ctas, uint64_t(num_sms) * 8)), 32 * NW, csmem, st, P, nj);
+  launch(row_base_kernel, P.trows, 256, 0, st, P);
+  launch(trow_plan_kernel, 1, 1024, 0, st, P);
+  launch(place_kernel<J, BWD>, unsigned(std::min<uint64_t>(ctas, uint64_t(num_sms) * 16)), 32 * NW, smem, st, P, nj);
   return cudaGetLastError();
 }
 
