@@ -287,6 +287,104 @@ __global__ void __launch_bounds__(256) hist_scan_kernel(uint32_t *hist, int G, u
   if (threadIdx.x == 0) digit_total[blockIdx.x] = tot;
 }
 
+// The whole depth sort of up to 6,144 pairs in one CTA: the keys of the pairs that are left (ids fit
+// 16 bits) stay in shared memory between the four passes, ranked as in sort_downsweep, each warp
+// over a contiguous part.  Bound by the latency of its steps: a frame of
+// 1,000 primitives took 92 us with the eight launches of the passes and 75 us with this one, of 4,096
+// 132 and 121, of 6,000 155 and 149; at 8,192 (16 items per thread) both took 173.
+constexpr int kSmallThreads = 512, kSmallWarps = kSmallThreads / 32, kSmallIPT = 12;
+constexpr int kSmallItems = kSmallThreads * kSmallIPT;
+constexpr size_t kSmallSmem = size_t(kSmallItems) * 6 + size_t(kSmallWarps) * 256 * 4;
+
+__global__ void __launch_bounds__(kSmallThreads) sort_small_kernel(SortPass p) {
+  await_previous();
+  extern __shared__ uint32_t s_small[];
+  uint32_t *s_key = s_small;                                               // [kSmallItems]
+  uint32_t(*s_cnt)[256] = reinterpret_cast<uint32_t(*)[256]>(s_key + kSmallItems);  // [kSmallWarps][256]
+  uint16_t *s_id = reinterpret_cast<uint16_t *>(s_cnt + kSmallWarps);      // [kSmallItems]
+  __shared__ uint32_t s_base[256];
+  __shared__ uint32_t s_ws[33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t m = min(p.count_max, uint32_t(kSmallItems));  // items before the pass
+  for (int shift = 0; shift < 32; shift += 8) {
+    const uint32_t rounds = (m + kSmallThreads - 1) / kSmallThreads, first = warp * (32 * rounds) + lane;
+    uint32_t key[kSmallIPT], id[kSmallIPT], off[kSmallIPT], vmask = 0;
+#pragma unroll
+    for (int r = 0; r < kSmallIPT; ++r) {
+      const uint32_t idx = first + r * 32;
+      const bool ok = r < rounds && idx < m;
+      key[r] = !ok ? kCulled : shift ? s_key[idx] : p.keys_in[idx];
+      id[r] = !ok ? 0u : shift ? s_id[idx] : idx;
+      if (ok && (shift || key[r] != kCulled)) vmask |= 1u << r;
+    }
+    for (int i = threadIdx.x; i < kSmallWarps * 256; i += kSmallThreads) (&s_cnt[0][0])[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSmallIPT; ++r) {
+      if (r >= rounds) break;
+      const bool valid = (vmask >> r) & 1u;
+      const uint32_t d = (key[r] >> shift) & 255u;
+      uint32_t peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+      for (int bit = 0; bit < 8; ++bit) {
+        const uint32_t bal = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
+        peers &= ((d >> bit) & 1u) ? bal : ~bal;
+      }
+      if (!valid) peers = 1u << lane;
+      const uint32_t c = valid ? s_cnt[warp][d] : 0u;
+      __syncwarp();
+      if (valid && lane == 31 - __clz(peers)) s_cnt[warp][d] = c + __popc(peers);
+      __syncwarp();
+      off[r] = c + __popc(peers & lt);
+    }
+    __syncthreads();
+    uint32_t run = 0;
+    if (threadIdx.x < 256) {
+#pragma unroll
+      for (int w = 0; w < kSmallWarps; ++w) {
+        const uint32_t c = s_cnt[w][threadIdx.x];
+        s_cnt[w][threadIdx.x] = run;
+        run += c;
+      }
+    }
+    uint32_t kept;
+    const uint32_t lower = block_excl_scan(run, s_ws, &kept);
+    if (threadIdx.x < 256) s_base[threadIdx.x] = lower;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSmallIPT; ++r) {
+      if (vmask & (1u << r)) {
+        const uint32_t d = (key[r] >> shift) & 255u, pos = s_base[d] + s_cnt[warp][d] + off[r];
+        s_key[pos] = key[r];
+        s_id[pos] = uint16_t(id[r]);
+      }
+    }
+    m = kept;
+    __syncthreads();
+  }
+  for (uint32_t j = threadIdx.x; j < m; j += kSmallThreads) {
+    const uint32_t v = s_id[j], ri = p.row_info[v];
+    uint32_t ty0 = ri & 0xFFu, cnt = ri >> 8;
+    if (cnt >= 255u || ty0 == 255u) {
+      const uint2 r = p.row_rect[v];
+      ty0 = r.x >> 16;
+      cnt = (r.y >> 16) - ty0 + 1;
+    }
+    p.keys_out[j] = ty0 | ((cnt - 1u) << 12) | ((v / p.n) << 24);
+    p.vals_out[j] = v;
+  }
+  if (threadIdx.x == 0) *p.d_total = m;
+}
+
+bool sort_is_small(uint64_t pairs) { return pairs <= uint64_t(kSmallItems); }
+
+cudaError_t launch_sort_small(const SortPass &p, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmallSmem));
+  if (e != cudaSuccess) return e;
+  return launch(sort_small_kernel, 1, kSmallThreads, kSmallSmem, st, p);
+}
+
 // One LSD pass: 8-bit digits for the depth sort, 4 or 6 bits for the split by view.  The grid
 // is at most one CTA per 2,048 items.  Up to kSortNoScan CTAs (32,768 items) every downsweep
 // CTA reads the counts of all of them instead of a scan kernel's offsets: two launches instead

@@ -203,7 +203,18 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   base.id_bits = 1;
   while (base.id_bits < 32 && (uint64_t(1) << base.id_bits) < uint64_t(VN)) ++base.id_bits;
   int cur = 0;
-  for (int pass = 0; pass < 4; ++pass) {
+  const bool small = sort_is_small(VN);
+  if (small) {
+    SortPass sp = base;
+    sp.keys_in = w.at<uint32_t>(w.L.depth);
+    sp.keys_out = w.at<uint32_t>(w.L.s1k[cur]);
+    sp.vals_out = w.at<uint32_t>(w.L.s1v[cur]);
+    sp.d_total = &ctr->n_visible;
+    sp.row_info = w.at<uint16_t>(w.L.rinfo);
+    sp.row_rect = w.at<uint2>(w.L.rect);
+    if ((e = launch_sort_small(sp, st)) != cudaSuccess) return e;
+  }
+  for (int pass = 0; pass < (small ? 0 : 4); ++pass) {
     SortPass sp = base;
     sp.keys_in = w.at<uint32_t>(pass == 0 ? w.L.depth : w.L.s1k[cur]);
     sp.vals_in = pass == 0 ? nullptr : w.at<uint32_t>(w.L.s1v[cur]);

@@ -404,6 +404,8 @@ void note_cuda_error(cudaError_t e);
 
 cudaError_t launch_preprocess(const PrepParams &P, int num_sms, cudaStream_t st);
 cudaError_t launch_sort_pass(SortPass p, cudaStream_t st);
+bool sort_is_small(uint64_t pairs);  // one kernel for the whole depth sort
+cudaError_t launch_sort_small(const SortPass &p, cudaStream_t st);  // row_info, row_rect and d_total set
 uint32_t place_cp_lo(int max_rows);
 uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows);
 cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st);
