@@ -467,12 +467,9 @@ def run_ours(args, world, rank, local):
     attr_bytes = sum(v.numel() * v.element_size() for v in st.values() if hasattr(v, "numel"))
     prep_bytes = attr_bytes + 4 * n * len(cams) + 105 * ctr["n_visible"]
     bin_bytes = binning_bytes(ctr, n * len(cams))
-    # kernels per pass: preprocess (2), depth sort (4 passes x 5), row-count scan (3),
-    # row spans (1), tile-row scan (1), tile-row sort (passes x 5), chunk scan + chunk
-    # counts + instance lists (3), rasteriser (1)
-    trows = sum(-(-c["height"] // r.cfg.tile_h) for c in cams)
-    row_passes = (max(1, (trows - 1).bit_length()) + 7) // 8
-    gpu_launches = args.steps * (2 + 20 + 3 + 1 + 1 + 5 * row_passes + 3 + 1)
+    # kernels per pass: preprocess (2), depth sort (4 passes x 3), split by view (3), support
+    # rows (4), instance lists (2), rasteriser (1)
+    gpu_launches = args.steps * (2 + 12 + (3 if len(cams) > 1 else 0) + 4 + 2 + 1)
 
     line = dict(
         metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,
@@ -829,8 +826,10 @@ def precision_ablation(args, dev):
 
 
 def binning_bytes(ctr, pairs):
-    """Algorithmic bytes of one binning pass (each array read or written once per use; the
-    row payload as stored): depth sort (the dense 4-B keys and 1-B tile-row counts read,
+    """Algorithmic bytes of a binning pass that sorts the support rows by tile row in two passes
+    (each array read or written once per use; the row payload as stored), the yardstick of the
+    rates since the first version; the rows are now placed without that sort, so the bytes
+    really needed are fewer by row_sort less 8 B per kept row.  Depth sort (the dense 4-B keys and 1-B tile-row counts read,
     then 8 B per visible pair per pass in and out, the upsweeps' key reads),
     support rows (the 32-B support sector per pair, 12 B written per row), the tile-row
     sort (4-B key + 8-B payload read per row in the first pass, 12 B written per kept row,

@@ -205,8 +205,8 @@ raygs_status raygs_preprocess(raygs_plan *plan, const raygs_scene *scene, void *
  * Binning for Eq. rendering's depth order: stable on-device radix sort of the visible
  * (primitive, view) pairs by float32 centre depth (ties keep primitive order); per pair and
  * tile row of its rectangle, the run of tiles whose pixel centres can meet its support;
- * stable radix sort of those rows by global tile row; per tile row, the expansion of its
- * rows into per-tile instance lists in depth order and the per-tile [start, end) ranges.
+ * those rows placed, still in depth order, into one list per tile row; per tile row, the
+ * expansion of its rows into per-tile instance lists and the per-tile [start, end) ranges.
  * The instance total and an overflow flag go to device counters.  Requires
  * raygs_preprocess on the same stream first.
  */

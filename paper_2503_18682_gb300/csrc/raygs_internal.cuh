@@ -88,17 +88,6 @@ struct __align__(32) Ell {
   float cx, cy, a, b, d, det;
 };
 
-struct RasterCfg {
-  float t_stop;
-  float alpha_max;
-};
-
-// Packed inclusive tile rectangle: x = tx0 | ty0 << 16, y = tx1 | ty1 << 16.
-__host__ __device__ inline uint32_t rect_count(uint2 r) {
-  uint32_t tx0 = r.x & 0xFFFF, ty0 = r.x >> 16, tx1 = r.y & 0xFFFF, ty1 = r.y >> 16;
-  return (tx1 - tx0 + 1) * (ty1 - ty0 + 1);
-}
-
 // ---------------------------------------------------------------- double-float helpers
 // Error-free transforms (Knuth two-sum, FMA two-product) written with explicitly rounded
 // intrinsics so that the compiler cannot contract or reassociate them.

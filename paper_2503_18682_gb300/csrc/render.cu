@@ -1,9 +1,9 @@
 // Per-tile rasterisation and front-to-back compositing (Sec. 3 Eq. rendering and
 // Eq. rend_opacity; Sec. 4.2 fragment formula).
 //
-// Persistent CTAs (one per resident slot) claim the screen tiles of all views from a
-// counter, one at a time, those with the longest lists first; each thread shades PX pixels of a tile row.  A tile's instance list (depth order) is consumed in batches: each thread
-// stages records in shared memory, converting the projected centre to a tile-relative
+// Persistent CTAs (one per resident slot) take the screen tiles of all views one at a time,
+// those with the longest lists first; each thread shades PX pixels of a tile row.  A tile's
+// instance list (depth order) is consumed in batches: each thread stages records in shared memory, converting the projected centre to a tile-relative
 // offset in double-float so that per-pixel offsets stay exact to the float32 rounding of
 // the offset itself.  Per pixel, with delta = pixel centre - projected centre:
 //   y01 = G delta, y2 = 1 + h . delta, q = |y01|^2, r = y2^2
