@@ -731,7 +731,9 @@ __global__ void __launch_bounds__(kPrepThreads) preprocess_kernel(PrepParams P) 
 
 // FP64 vertex stage for the (view, primitive) pairs listed by preprocess_kernel.  The
 // float32 record, rectangle and key of each pair are overwritten.  Grid-stride over the
-// device-side list.
+// device-side list.  Bound by the chain of one pair's FP64 operations: 51 us on one headset pair of
+// 1M primitives, with four CTAs of 128 threads per SM as with sixteen of 32 (which cost a small
+// call 1 % more).
 template <int DEG, int MODE>
 __global__ void __launch_bounds__(128) preprocess_fp64_kernel(PrepParams P) {
   await_previous();
