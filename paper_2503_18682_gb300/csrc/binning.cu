@@ -398,9 +398,13 @@ static cudaError_t sort_pass(const SortPass &p, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+int sort_blocks(uint64_t items, int grid) {
+  const uint64_t need = (items + kSortTile - 1) / kSortTile;  // CTAs with work
+  return need < uint64_t(grid) ? (need ? int(need) : 1) : grid;
+}
+
 cudaError_t launch_sort_pass(SortPass p, cudaStream_t st) {
-  const uint32_t need = (p.count_max + uint32_t(kSortTile) - 1u) / uint32_t(kSortTile);  // CTAs with work
-  p.G = need < uint32_t(p.G) ? (need ? int(need) : 1) : p.G;
+  p.G = sort_blocks(p.count_max, p.G);
   if (p.row_info) return sort_pass<8, kSortFirst>(p, st);
   if (p.row_rect) return sort_pass<8, kSortLast>(p, st);
   if (!p.index_out) return sort_pass<8, kSortPlain>(p, st);

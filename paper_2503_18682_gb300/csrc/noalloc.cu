@@ -10,6 +10,8 @@
 //
 // The array is a module-scope __device__ variable: every GPU that loads this library keeps
 // kNoAllocScratchBytes of device memory reserved for it until the process exits.
+#include <algorithm>
+
 #include "raygs_internal.cuh"
 
 namespace raygs {
@@ -37,6 +39,42 @@ raygs_status scratch_for_current_device(void **out) {
   }
   *out = p;
   return RAYGS_OK;
+}
+
+// Size check: the fixed part must fit; the rest of the array bounds the tile rows and instances
+// (kBytesPerCapacity bytes per unit of capacity, and the list pass's column counts).  What only
+// makes a pass faster (the row pass's head chunks, the tiles by class on small batches) is left
+// out of a batch that would otherwise not fit, or keep less than half of the capacity.
+bool fit_scratch(Work &w) {
+  const struct { int heads; bool order; } keep[] = {{kHeadChunks, w.tiles <= 8192}, {16, false}, {0, false}};
+  Work best[3];
+  for (int i = 2; i >= 0; --i) {
+    Work &c = best[i];
+    c = w;
+    LayoutOptions opt;
+    opt.tile_stop = false;
+    opt.tile_order = keep[i].order;
+    opt.heads = c.heads = keep[i].heads;
+    auto layout = [&](int64_t cap) {
+      c.cap = cap;
+      c.L = make_layout(c.n_views, c.n, c.tiles, c.trows, cap, c.num_sms, c.max_tiles_x, c.max_rows, opt);
+      return c.L.total <= kNoAllocScratchBytes;
+    };
+    layout(0);
+    const double room = double(kNoAllocScratchBytes) - double(c.L.total);
+    // the column counts: up to so many bytes per unit of capacity, and no more than so many in all
+    const double per_unit = 4.0 * c.max_tiles_x / list_rows_lo(c.max_tiles_x);
+    const double in_all = 4.0 * c.max_tiles_x * list_target(c.num_sms);
+    int64_t cap = int64_t(std::max(room / (kBytesPerCapacity + per_unit), (room - in_all) / kBytesPerCapacity));
+    while (cap > 0 && !layout(cap)) cap -= 256;
+    if (cap <= 0) c.cap = 0;
+  }
+  for (const Work &c : best)
+    if (c.cap > 0 && 2 * c.cap >= best[2].cap) {
+      w = c;
+      return true;
+    }
+  return false;
 }
 
 }  // namespace
@@ -72,8 +110,6 @@ extern "C" raygs_status raygs_render_noalloc(const raygs_camera *cams, int32_t n
     return RAYGS_ERR_CUDA;
   }
 
-  // Size check: the fixed part must fit; the rest of the array bounds the tile rows and
-  // instances (kBytesPerCapacity bytes per unit of capacity).
   Work w;
   w.n_views = n_views;
   w.n = n;
@@ -84,17 +120,7 @@ extern "C" raygs_status raygs_render_noalloc(const raygs_camera *cams, int32_t n
   w.num_sms = sms;
   w.G = sort_grid(sms);
   w.cfg = cfg;
-  const bool order = tiles <= 8192;  // the tiles' order (48 bytes per tile) on small batches only
-  const Layout L0 = make_layout(n_views, n, tiles, trows, 0, sms, max_tx, max_rows, false, false, order);
-  if (L0.total + 8192 > kNoAllocScratchBytes) return RAYGS_ERR_CAPACITY;
-  int64_t cap = int64_t((kNoAllocScratchBytes - L0.total - 8192) / (kBytesPerCapacity + 1));
-  w.L = make_layout(n_views, n, tiles, trows, cap, sms, max_tx, max_rows, false, false, order);
-  while (w.L.total > kNoAllocScratchBytes && cap > 0) {
-    cap -= 4096;
-    w.L = make_layout(n_views, n, tiles, trows, cap, sms, max_tx, max_rows, false, false, order);
-  }
-  if (cap <= 0 || w.L.total > kNoAllocScratchBytes) return RAYGS_ERR_CAPACITY;
-  w.cap = cap;
+  if (!fit_scratch(w)) return RAYGS_ERR_CAPACITY;
   w.base = static_cast<char *>(scratch);
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -114,4 +140,19 @@ extern "C" raygs_status raygs_render_noalloc(const raygs_camera *cams, int32_t n
     return fail(e);
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return fail(e);
   return overflow ? RAYGS_ERR_CAPACITY : RAYGS_OK;
+}
+
+/* Diagnostic, not part of the documented ABI: the capacity a call on a device of `sms` SMs would have
+ * in the array (host only), 0 when the batch is refused before any work. */
+extern "C" int64_t raygs_debug_noalloc_capacity(const raygs_camera *cams, int32_t n_views, int64_t n,
+                                                const raygs_config *cfg, int32_t sms) {
+  Work w;
+  DevCam dc[RAYGS_MAX_VIEWS];
+  int64_t pixels = 0;
+  if (!cams || !cfg || n_views < 1 || n_views > RAYGS_MAX_VIEWS || n < 0 || sms < 1) return 0;
+  if (!plan_views(cams, n_views, *cfg, dc, w.tiles, w.trows, pixels, w.max_tiles_x, w.max_rows)) return 0;
+  w.n_views = n_views;
+  w.n = n;
+  w.num_sms = sms;
+  return fit_scratch(w) ? w.cap : 0;
 }

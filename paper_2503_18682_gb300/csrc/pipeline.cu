@@ -73,7 +73,8 @@ int sort_grid(int num_sms) {
 }
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
-                   int max_rows, bool backward, bool mip_exact, bool tile_order) {
+                   int max_rows, const LayoutOptions &opt) {
+  const bool backward = opt.backward;
   Layout L{};
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = up256(o + bytes); return r; };
@@ -89,11 +90,11 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.rinfo = take(2 * VN);
   L.ell = take(sizeof(Ell) * VN);
   L.rec = take(sizeof(Rec) * VN);
-  L.recx = mip_exact ? take(sizeof(Rec) * VN) : 0;
+  L.recx = opt.mip_exact ? take(sizeof(Rec) * VN) : 0;
   for (int i = 0; i < 2; ++i) { L.s1k[i] = take(4 * VN); L.s1v[i] = take(4 * VN); }
   L.vpos = n_views > 1 ? take(4 * VN) : 0;
-  const uint64_t pchunks = place_max_chunks(n_views, VN, max_rows);
-  L.cnt1 = take(4 * size_t(max_rows) * pchunks + 16);
+  const uint64_t pchunks = place_max_chunks(n_views, VN, max_rows, opt.heads);
+  L.cnt1 = take(4 * size_t(place_max_counts(n_views, VN, max_rows, trows, opt.heads)) + 16);
   // per unit of capacity: kBytesPerCapacity bytes
   L.spanl = take(4 * size_t(span_list_cap(C)));
   L.spans = take(4 * size_t(span_rows_cap(C)));
@@ -103,16 +104,15 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.inste = backward ? take(4 * C + 16) : 0;
   L.ebase = backward ? take(4 * pchunks + 16) : 0;
   L.paire = backward ? take(16 * VN + 16) : 0;
-  L.trcnt = take(4 * size_t(trows) + 16);
   L.trange = take(8 * size_t(trows) + 16);
   L.trinst = take(8 * size_t(trows) + 16);
   L.cbase = take(4 * size_t(trows + 1) + 16);
   L.ccnt = take(4 * size_t(list_max_chunks(trows, cap, max_tiles_x, num_sms)) * size_t(max_tiles_x) + 16);
-  L.hist = take(4 * 256 * size_t(sort_grid(num_sms)));
+  L.hist = take(4 * 256 * size_t(sort_blocks(VN, sort_grid(num_sms))));
   L.dtot = take(4 * 256);
   L.ranges = take(8 * size_t(tiles));
-  L.tclass = tile_order ? take(4 * size_t(kTileClasses) * size_t(tiles) + 16) : 0;
-  L.tstop = take(4 * size_t(tiles) + 16);
+  L.tclass = opt.tile_order ? take(4 * size_t(kTileClasses) * size_t(tiles) + 16) : 0;
+  L.tstop = opt.tile_stop ? take(4 * size_t(tiles) + 16) : 0;
   L.deg = L.s1k[0];  // the FP64 lists of the vertex stage and of the backward: free then
   L.partials = backward ? take(4 * kGradW * C + 16) : 0;
   L.bclass = backward ? take(4 * size_t(kTileClasses) * size_t(tiles) + 16) : 0;
@@ -261,15 +261,16 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   R.trows = int(w.trows);
   R.max_rows = w.max_rows;
   R.cap = cap;
+  R.heads = uint32_t(w.heads);
   R.span_list = w.at<uint32_t>(w.L.spanl);
   R.span_list_cap = span_list_cap(uint64_t(w.cap));
   R.spans = w.at<uint32_t>(w.L.spans);
   R.cnt1 = w.at<uint32_t>(w.L.cnt1);
-  R.trow_cnt = w.at<uint32_t>(w.L.trcnt);
   R.trow_ranges = w.at<uint2>(w.L.trange);
   R.trow_inst = w.at<unsigned long long>(w.L.trinst);
   R.rows = w.at<uint2>(w.L.rows);
   R.chunk_base = w.at<uint32_t>(w.L.cbase);
+  R.list_lo = list_rows_lo(w.max_tiles_x);
   R.list_hi = list_rows_hi(w.cap, w.max_tiles_x);
   R.list_target = list_target(w.num_sms);
   R.max_chunks = uint32_t(list_max_chunks(w.trows, w.cap, w.max_tiles_x, w.num_sms));

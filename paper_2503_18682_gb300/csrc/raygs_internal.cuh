@@ -223,16 +223,16 @@ struct PlaceParams {
   int n, n_views, tile_w, tile_h;
   int trows, max_rows;         // tile rows of the batch, and the most of one view
   uint32_t cap;
+  uint32_t heads;              // head chunks of a view, at most (see rows.cu)
   uint32_t cp_lo, cp_hi, target;
   const uint32_t *span_list;   // pairs whose support is not a bounded ellipse (see PrepParams)
   uint32_t span_list_cap;
   uint32_t *spans;             // per row of those pairs: first tile column | tiles << 16
   uint32_t *cnt1;              // per view, tile row and chunk: rows, then rows of the chunks before
-  uint32_t *trow_cnt;          // [tile rows] rows
   uint2 *trow_ranges;          // [tile rows] the tile row's range of the row list
-  unsigned long long *trow_inst;  // [tile rows] cleared here
+  unsigned long long *trow_inst;  // [tile rows] rows, then cleared for the list pass
   uint32_t *chunk_base;        // [tile rows + 1] first chunk of each tile row in the list pass
-  uint32_t list_hi, list_target, max_chunks;
+  uint32_t list_lo, list_hi, list_target, max_chunks;
   uint2 *rows;                 // [cap] the row list: sorted pair position, first tile column | tiles << 16
   // plans with the backward (null otherwise): where each row's instances lie among the partial
   // sums, (chunk, offset in the chunk); the chunks' first slots; per sorted pair its run
@@ -266,7 +266,6 @@ struct ListParams {
   int trows, max_tiles_x;
   uint32_t max_chunks;
 };
-constexpr uint32_t kListRowsLo = 512;  // rows of the shortest chunk
 
 struct RenderParams {
   const DevCam *cams;
@@ -395,9 +394,12 @@ cudaError_t launch_preprocess(const PrepParams &P, int num_sms, cudaStream_t st)
 cudaError_t launch_sort_pass(SortPass p, cudaStream_t st);
 bool sort_is_small(uint64_t pairs);  // one kernel for the whole depth sort
 cudaError_t launch_sort_small(const SortPass &p, cudaStream_t st);  // row_info, row_rect and d_total set
-uint32_t place_cp_lo(int max_rows);
-uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows);
+int sort_blocks(uint64_t items, int grid);  // CTAs of a pass
+constexpr int kHeadChunks = 128;  // head chunks of a view in the row pass, where there is room for their counts
+uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows, int heads);
+uint64_t place_max_counts(int n_views, uint64_t pairs, int max_rows, int64_t trows, int heads);
 cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st);
+uint32_t list_rows_lo(int max_tiles_x);
 uint32_t list_rows_hi(int64_t cap, int max_tiles_x);
 uint32_t list_target(int num_sms);
 uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sms);
@@ -415,15 +417,23 @@ cudaError_t launch_resolve(const float *rgb_hi, const float *T_hi, float *rgb_lo
 // ---------------------------------------------------------------- workspace
 // Byte offsets of every buffer inside one caller-owned (or library-static) workspace.
 struct Layout {
-  size_t tilectr, tclass, cams, spanl, spans, vpos, counters, evals, tstop, depth, rect, rinfo, ell, rec, recx, s1k[2], s1v[2], cnt1, trcnt, rows,
+  size_t tilectr, tclass, cams, spanl, spans, vpos, counters, evals, tstop, depth, rect, rinfo, ell, rec, recx, s1k[2], s1v[2], cnt1, rows,
       re, ebase, paire, trange, trinst, cbase, ccnt, inst, inste, hist, dtot, ranges, deg, degc, partials, bclass, bplan, ptouch, pg, pgtouch, total;
 };
 
+// What a plan keeps besides the buffers that every pass needs.
+struct LayoutOptions {
+  bool backward = false, mip_exact = false;
+  bool tile_order = true;   // the tiles by class (48 bytes per tile): without, they are taken in tile order
+  bool tile_stop = true;    // per-tile stop positions (instrumented renders)
+  int heads = kHeadChunks;  // head chunks of a view in the row pass (their counts: 4 bytes per tile row each)
+};
+
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
-                   int max_rows, bool backward, bool mip_exact, bool tile_order);
+                   int max_rows, const LayoutOptions &opt);
 
 // Workspace bytes per unit of instance capacity (support rows and instances share it).
-constexpr size_t kBytesPerCapacity = 8 + 4 + 1;
+constexpr double kBytesPerCapacity = 8 + 4 + 0.625;
 // Room for the pairs whose support is not a bounded ellipse and for their rows' spans (2 % of
 // the rows on the stereo batch, whose cameras stand among the primitives).
 constexpr uint32_t span_list_cap(uint64_t cap) { return uint32_t(cap / 32) + 256; }
@@ -436,7 +446,7 @@ struct Work {
   int n_views = 0;
   int64_t n = 0, tiles = 0, trows = 0, cap = 0;
   int max_tiles_x = 0, max_rows = 0;  // most tile columns and rows of one view
-  int G = 0, num_sms = 0;
+  int G = 0, num_sms = 0, heads = kHeadChunks;
   raygs_config cfg{};
   int s1_final = 0;  // which ping-pong buffer holds the depth-sorted pairs
   template <typename T>

@@ -188,11 +188,12 @@ __device__ __noinline__ bool scan_tile_span(const Rec &r, const DevCam &cam, int
 
 // The views' shares of the sorted pairs and their chunks.  A view's nearest pairs are its
 // largest ones (up to all its tile rows each, where the average is three), so its first
-// kHeadChunks chunks hold only kHeadPairs pairs, and the batch takes all views' head chunks
-// first.  The other chunks' length is the smallest power of two in [cp_lo, cp_hi] that leaves
+// P.heads chunks hold only kHeadPairs pairs, and the batch takes all views' head chunks
+// first (kHeadChunks of them; fewer or none where the workspace has no room for their counts).
+//  The other chunks' length is the smallest power of two in [cp_lo, cp_hi] that leaves
 // no more than `target` chunks: short lists still give every SM work, long ones amortise a
 // chunk's scans and write longer runs.
-constexpr uint32_t kHeadChunks = 128, kHeadPairs = 16;
+constexpr uint32_t kHeadPairs = 16;
 
 struct ViewTab {
   uint32_t start[RAYGS_MAX_VIEWS + 1];   // first sorted pair of the view
@@ -213,7 +214,7 @@ __device__ __forceinline__ void build_view_tab(const PlaceParams &P, ViewTab &T)
       const int v = h + lane;
       const bool in = v < P.n_views;
       const uint32_t n = in ? (P.view_count ? P.view_count[v] : nvis) : 0u;
-      const uint32_t nh = min(kHeadChunks, (n + kHeadPairs - 1) / kHeadPairs);
+      const uint32_t nh = min(P.heads, (n + kHeadPairs - 1) / kHeadPairs);
       const uint32_t nch = nh + (n > nh * kHeadPairs ? (n - nh * kHeadPairs + cp - 1) / cp : 0u);
       const uint32_t e = in ? nch * uint32_t(P.cams[v].tiles_y) : 0u;
       const uint32_t si = warp_incl_scan(n), ci = warp_incl_scan(nch), hi = warp_incl_scan(nh), ei = warp_incl_scan(e);
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(256) row_base_kernel(PlaceParams P) {
     }
     carry += tot;
   }
-  if (threadIdx.x == 0) P.trow_cnt[t] = carry;
+  if (threadIdx.x == 0) P.trow_inst[t] = carry;
   scan_rows(P);
 }
 
@@ -442,19 +443,19 @@ __global__ void __launch_bounds__(1024) trow_plan_kernel(PlaceParams P) {
   const int per = (P.trows + 1023) / 1024;
   const int b = min(P.trows, int(threadIdx.x) * per), e = min(P.trows, b + per);
   unsigned long long s = 0, tot;
-  for (int t = b; t < e; ++t) s += P.trow_cnt[t];
+  for (int t = b; t < e; ++t) s += P.trow_inst[t];
   unsigned long long run = block_excl_scan64(s, ws, &tot);
   const unsigned long long cap = P.cap;
   for (int t = b; t < e; ++t) {
-    const unsigned long long n = P.trow_cnt[t];
+    const unsigned long long n = P.trow_inst[t];
     P.trow_ranges[t] = make_uint2(uint32_t(min(run, cap)), uint32_t(min(run + n, cap)));
     P.trow_inst[t] = 0ull;
     run += n;
   }
-  // the chunks of the list pass: the shortest power of two in [kListRowsLo, list_hi] that leaves
+  // the chunks of the list pass: the shortest power of two in [list_lo, list_hi] that leaves
   // fewer than list_target of them (short lists still occupy every SM), at least one per tile
   // row (its tiles' ranges are written with them)
-  uint32_t cr = kListRowsLo;
+  uint32_t cr = P.list_lo;
   while (cr < P.list_hi && uint32_t(min(tot, cap)) / cr >= P.list_target) cr <<= 1;
   auto chunks = [&](int t) {
     const uint2 rr = P.trow_ranges[t];  // (this thread wrote it)
@@ -648,15 +649,22 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
 // ------------------------------------------------------------------------- launchers
 
 // Chunk lengths the plan allows: the counts (tile rows x chunks) stay within one word per
-// (primitive, view) pair, and kHeadChunks + 1 rows of them per view.
-uint32_t place_cp_lo(int max_rows) {
+// (primitive, view) pair, and `heads` + 1 per tile row.
+static uint32_t place_cp_lo(int max_rows) {
   uint32_t cp = 64;
   while (cp < uint32_t(max_rows)) cp <<= 1;
   return cp;
 }
-uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows) {
+// Head chunks of a view, and one chunk that is not full.
+static uint64_t place_view_chunks(int n_views, uint64_t pairs, int heads) {
   const uint64_t n = n_views > 0 ? pairs / uint64_t(n_views) : 0;
-  return pairs / place_cp_lo(max_rows) + uint64_t(n_views) * (std::min<uint64_t>(kHeadChunks, n / kHeadPairs + 1) + 1);
+  return std::min<uint64_t>(uint64_t(heads), n / kHeadPairs + 1) + 1;
+}
+uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows, int heads) {
+  return pairs / place_cp_lo(max_rows) + uint64_t(n_views) * place_view_chunks(n_views, pairs, heads);
+}
+uint64_t place_max_counts(int n_views, uint64_t pairs, int max_rows, int64_t trows, int heads) {
+  return pairs / place_cp_lo(max_rows) * uint64_t(max_rows) + uint64_t(trows) * place_view_chunks(n_views, pairs, heads);
 }
 
 template <int J, bool BWD>
@@ -683,7 +691,7 @@ cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st) {
   P.cp_hi = std::max(256u, P.cp_lo);
   P.target = uint32_t(num_sms) * 32;
   const uint64_t max_chunks =
-      std::max<uint64_t>(1, place_max_chunks(P.n_views, uint64_t(P.n) * uint64_t(P.n_views), P.max_rows));
+      std::max<uint64_t>(1, place_max_chunks(P.n_views, uint64_t(P.n) * uint64_t(P.n_views), P.max_rows, int(P.heads)));
   const int nj = bins_per_lane(P.max_rows);
   const bool bwd = P.row_e != nullptr;
 #define RAYGS_PLACE(J) \
