@@ -286,7 +286,12 @@ cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int bat
   // SM).  500k primitives at 1280x720 (1.5 tiles per slot) 130 against 174 us whole, 1440x810 (1.9)
   // 141 against 168, 1600x900 (2.3) 154 against 171 (2M primitives: 211 against 210); 1920x1080
   // (3.4) 194 against 187, 2560x1440 (5.9) 292 against 259.
-  const bool parts = 2 * int64_t(P.n_tiles) * tile_w * tile_h <= 5 * int64_t(num_sms) * 16 * 256;
+  // On 8x8 tiles, whose parts are the tiles themselves with one instead of two pixels per thread, up to
+  // 0.75: 500k primitives at 800x450 (0.59) 83 against 95 us whole, 880x495 (0.70) 91 against 94, 960x540
+  // (0.84) 99 against 95, 1280x720 137 against 115, 1600x900 188 against 149.  (16x8 and 32x16 tiles at
+  // 1440x810: 150 against 142, 169 against 339.)
+  const int64_t area = int64_t(P.n_tiles) * tile_w * tile_h, slots = int64_t(num_sms) * 16 * 256;
+  const bool parts = tile_w * tile_h <= 64 ? 4 * area <= 3 * slots : 2 * area <= 5 * slots;
 #define RAYGS_RENDER_CASE(TW, TH, PX, NBF)                                                       \
   if (tile_w == TW && tile_h == TH && batch_records == NBF)                                     \
     return gs ? run_render<TW, TH, PX, NBF, 1>(P, num_sms, count, parts, st)                    \
