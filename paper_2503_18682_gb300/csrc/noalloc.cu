@@ -41,8 +41,7 @@ raygs_status scratch_for_current_device(void **out) {
   return RAYGS_OK;
 }
 
-// Size check: the fixed part must fit; the rest of the array bounds the tile rows and instances
-// (kBytesPerCapacity bytes per unit of capacity, and the list pass's column counts).  What only
+// Size check: the fixed part must fit; the rest of the array bounds the tile rows and instances.  What only
 // makes a pass faster (the row pass's head chunks, the tiles by class on small batches) is left
 // out of a batch that would otherwise not fit, or keep less than half of the capacity.
 bool fit_scratch(Work &w) {
@@ -53,6 +52,7 @@ bool fit_scratch(Work &w) {
     c = w;
     LayoutOptions opt;
     opt.tile_stop = false;
+    opt.bin_once = true;
     opt.tile_order = keep[i].order;
     opt.heads = c.heads = keep[i].heads;
     auto layout = [&](int64_t cap) {

@@ -96,10 +96,10 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   const uint64_t pchunks = place_max_chunks(n_views, VN, max_rows, opt.heads);
   L.cnt1 = take(4 * size_t(place_max_counts(n_views, VN, max_rows, trows, opt.heads)) + 16);
   // per unit of capacity: kBytesPerCapacity bytes
-  L.spanl = take(4 * size_t(span_list_cap(C)));
-  L.spans = take(4 * size_t(span_rows_cap(C)));
   L.rows = take(8 * C + 16);
+  L.spanl = opt.bin_once ? L.rows + 4 * C : take(4 * size_t(span_list_cap(VN, C)));
   L.inst = take(4 * C + 16);
+  L.spans = L.inst;  // read by the row pass, before the lists are written
   L.re = backward ? take(8 * C + 16) : 0;
   L.inste = backward ? take(4 * C + 16) : 0;
   L.ebase = backward ? take(4 * pchunks + 16) : 0;
@@ -178,8 +178,8 @@ cudaError_t run_preprocess(Work &w, const raygs_scene &scene, cudaStream_t st) {
   P.recx = w.L.recx ? w.at<Rec>(w.L.recx) : nullptr;
   P.counters = w.at<Counters>(w.L.counters);
   P.span_list = w.at<uint32_t>(w.L.spanl);
-  P.span_list_cap = span_list_cap(uint64_t(w.cap));
-  P.span_cap = span_rows_cap(uint64_t(w.cap));
+  P.span_list_cap = span_list_cap(uint64_t(w.n_views) * uint64_t(w.n), uint64_t(w.cap));
+  P.span_cap = uint32_t(w.cap);
   P.deg_list = w.at<uint32_t>(w.L.deg);
   P.deg_count = w.at<uint32_t>(w.L.degc);
   return launch_preprocess(P, w.num_sms, st);
@@ -263,8 +263,9 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   R.cap = cap;
   R.heads = uint32_t(w.heads);
   R.span_list = w.at<uint32_t>(w.L.spanl);
-  R.span_list_cap = span_list_cap(uint64_t(w.cap));
+  R.span_list_cap = span_list_cap(VN, cap);
   R.spans = w.at<uint32_t>(w.L.spans);
+  R.scan = w.at<uint32_t>(w.L.rows);
   R.cnt1 = w.at<uint32_t>(w.L.cnt1);
   R.trow_ranges = w.at<uint2>(w.L.trange);
   R.trow_inst = w.at<unsigned long long>(w.L.trinst);

@@ -496,7 +496,7 @@ __device__ __forceinline__ void write_record_mipx(const PrepParams &P, int64_t i
 
 __device__ __forceinline__ void write_record(const PrepParams &P, int64_t idx, const DevCam &cam,
                                              const df muc[3], const StageOut &so, const float rgb[3],
-                                             float z, bool write_key) {
+                                             float z, bool write_key, bool last) {
   df X = df_div(muc[0], muc[2]);
   df Yv = df_div(muc[1], muc[2]);
   df u = df_add(df_mul_f(X, cam.fx), df{cam.cx, 0.f});
@@ -513,13 +513,13 @@ __device__ __forceinline__ void write_record(const PrepParams &P, int64_t idx, c
   e.cx = u.hi + so.dc0;
   e.cy = v.hi + so.dc1;
   e.a = so.M00; e.b = so.M01; e.d = so.M11; e.det = so.det;
-  if (!(so.M00 > 0.f)) {  // listed, with a place for its rows' spans (see PlaceParams)
+  if (last && !(so.M00 > 0.f)) {  // listed, with a place for its rows' spans (see PlaceParams)
     const uint32_t rows = uint32_t(so.ty1 - so.ty0 + 1);
-    const uint32_t base = atomicAdd(&P.counters->n_span_rows, rows);
+    const unsigned long long base = atomicAdd(&P.counters->n_span_rows, (unsigned long long)rows);
     const uint32_t i = atomicAdd(&P.counters->n_unbounded, 1u);
-    const bool room = i < P.span_list_cap && base < P.span_cap && rows <= P.span_cap - base;
+    const bool room = i < P.span_list_cap && base + rows <= P.span_cap;
     if (i < P.span_list_cap) P.span_list[i] = room ? uint32_t(idx) : kCulled;
-    e.cx = __uint_as_float(room ? base : kCulled);
+    e.cx = __uint_as_float(room ? uint32_t(base) : kCulled);
   }
   P.ell[idx] = e;
   // the rectangle also in its own compact array, and its tile rows in two bytes (see above)
@@ -717,9 +717,10 @@ __global__ void __launch_bounds__(kPrepThreads) preprocess_kernel(PrepParams P) 
       float rgb[3];
       sh_colour<DEG>(s_sh + tt * SHP, dx * dn, dy * dn, dz * dn, rgb);
       // (the cull pass wrote this pair's key)
+      const bool fp64 = s_deg[tt] && (P.fp64_degenerate == 2 || so.illcond);  // written again by the FP64 kernel
       if (MODE == kStageExact) write_record_mipx(P, idx, cam, muc, so, mxo, rgb, z, false);
-      else write_record(P, idx, cam, muc, so, rgb, z, false);
-      if (s_deg[tt] && (P.fp64_degenerate == 2 || so.illcond)) {
+      else write_record(P, idx, cam, muc, so, rgb, z, false, !fp64);
+      if (fp64) {
         const uint32_t slot = atomicAdd(P.deg_count, 1u);
         P.deg_list[slot] = uint32_t(idx);
       }
@@ -771,7 +772,7 @@ __global__ void __launch_bounds__(128) preprocess_fp64_kernel(PrepParams P) {
     float rgb[3];
     sh_colour<DEG>(coef, dx * dn, dy * dn, dz * dn, rgb);
     if (MODE == kStageExact) write_record_mipx(P, idx, cam, muc, so, mxo, rgb, z, true);
-    else write_record(P, idx, cam, muc, so, rgb, z, true);
+    else write_record(P, idx, cam, muc, so, rgb, z, true, true);
   }
 }
 

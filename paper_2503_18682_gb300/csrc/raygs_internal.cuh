@@ -53,8 +53,8 @@ struct Counters {
   unsigned long long n_nonfinite;
   uint32_t n_partials;      // partial-sum slots handed out (plans with the backward)
   uint32_t n_rows_kept;     // support rows with at least one tile
-  uint32_t n_unbounded;     // pairs whose support is not a bounded ellipse, and their rows
-  uint32_t n_span_rows;
+  unsigned long long n_span_rows;  // rows of the pairs whose support is not a bounded ellipse,
+  uint32_t n_unbounded;            // and those pairs
   uint32_t n_scan;          // rows of those pairs that have to be tested tile by tile
   uint32_t chunk_rows;      // rows per chunk of the list pass
   uint32_t lists_done;      // CTAs of list_count_kernel that have finished (0 between launches)
@@ -81,7 +81,7 @@ __device__ __forceinline__ int tile_class_of(uint32_t len) {
 // rounding), det = ad - b^2.  a < 0 marks a support that is not a bounded ellipse in the
 // image (or is too ill-conditioned in float32): binning then bounds its rows from the pair's
 // record (cx holds, as bits, the pair's first slot among the spans, kCulled when there was no
-// room: its rows then keep the whole rectangle); a = -2 keeps every tile of the rectangle (the
+// room, which only rows beyond the capacity bring about); a = -2 keeps every tile of the rectangle (the
 // exact anti-aliasing records hold no conic).
 struct __align__(32) Ell {
   uint32_t r0, r1;  // tx0 | ty0 << 16, tx1 | ty1 << 16
@@ -227,6 +227,7 @@ struct PlaceParams {
   uint32_t cp_lo, cp_hi, target;
   const uint32_t *span_list;   // pairs whose support is not a bounded ellipse (see PrepParams)
   uint32_t span_list_cap;
+  uint32_t *scan;              // [cap] spans left to be tested tile by tile (in the first half of rows)
   uint32_t *spans;             // per row of those pairs: first tile column | tiles << 16
   uint32_t *cnt1;              // per view, tile row and chunk: rows, then rows of the chunks before
   uint2 *trow_ranges;          // [tile rows] the tile row's range of the row list
@@ -426,18 +427,20 @@ struct LayoutOptions {
   bool backward = false, mip_exact = false;
   bool tile_order = true;   // the tiles by class (48 bytes per tile): without, they are taken in tile order
   bool tile_stop = true;    // per-tile stop positions (instrumented renders)
+  bool bin_once = false;    // one binning per vertex stage: what it reads of that need not outlast it
   int heads = kHeadChunks;  // head chunks of a view in the row pass (their counts: 4 bytes per tile row each)
 };
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
                    int max_rows, const LayoutOptions &opt);
 
-// Workspace bytes per unit of instance capacity (support rows and instances share it).
-constexpr double kBytesPerCapacity = 8 + 4 + 0.625;
-// Room for the pairs whose support is not a bounded ellipse and for their rows' spans (2 % of
-// the rows on the stereo batch, whose cameras stand among the primitives).
-constexpr uint32_t span_list_cap(uint64_t cap) { return uint32_t(cap / 32) + 256; }
-constexpr uint32_t span_rows_cap(uint64_t cap) { return uint32_t(cap / 8) + 1024; }
+// Workspace bytes per unit of instance capacity (support rows and instances share it), besides the
+// column counts of the list pass and the list below.
+constexpr size_t kBytesPerCapacity = 8 + 4;
+// Room for the pairs whose support is not a bounded ellipse: each has a row at least, so that none is
+// left out unless the rows overflow the capacity.  Their rows' spans lie where the instances come
+// later, one word per unit of capacity.
+constexpr uint32_t span_list_cap(uint64_t pairs, uint64_t cap) { return uint32_t(pairs < cap ? pairs : cap); }
 
 // A bound workspace and the sizes it was laid out for.
 struct Work {

@@ -292,7 +292,7 @@ __device__ __forceinline__ void unbounded_spans(const PlaceParams &P) {
     if (pair == kCulled) continue;
     const Ell e = P.ell[pair];
     const uint32_t base = __float_as_uint(e.cx);
-    if (e.a > 0.f || base == kCulled) continue;  // redone in FP64 since, as a bounded ellipse
+    if (base == kCulled) continue;
     const Rec &rec = P.rec[pair];
     const DevCam &cam = P.cams[pair / uint32_t(P.n)];
     const int tx0 = e.r0 & 0xFFFF, ty0 = e.r0 >> 16, tx1 = e.r1 & 0xFFFF, rows = int(e.r1 >> 16) - ty0 + 1;
@@ -302,13 +302,16 @@ __device__ __forceinline__ void unbounded_spans(const PlaceParams &P) {
       const float yb = float(min((ty0 + r + 1) * P.tile_h, cam.H)) - 0.5f;
       int a0 = 0, b0 = -1, state = 0;
       if (r < rows) state = support_tile_span(rec, cam, P.tile_w, ya, yb, tx0, tx1, a0, b0);
-      if (state < 0) {  // left to scan_rows (the row list is free until place_kernel)
+      uint32_t span = state ? uint32_t(a0) | (uint32_t(b0 - a0 + 1) << 16) : 0u;
+      if (state < 0) {  // left to scan_rows; until then the span holds the pair's place in the list
+        span = uint32_t(tx0) | (uint32_t(tx1 - tx0 + 1) << 16);
         const uint32_t j = atomicAdd(&P.counters->n_scan, 1u);
-        a0 = tx0;
-        b0 = tx1;
-        if (j < P.cap) P.rows[j] = make_uint2(pair, uint32_t(r));
+        if (j < P.cap) {  // (always: there are no more spans)
+          P.scan[j] = base + uint32_t(r);
+          span = uint32_t(u / parts);
+        }
       }
-      if (r < rows) P.spans[base + r] = state ? uint32_t(a0) | (uint32_t(b0 - a0 + 1) << 16) : 0u;
+      if (r < rows) P.spans[base + r] = span;
     }
   }
 }
@@ -318,17 +321,16 @@ __device__ __forceinline__ void scan_rows(const PlaceParams &P) {
   const uint32_t n = min(P.counters->n_scan, P.cap);
   const uint32_t warps = gridDim.x * (blockDim.x >> 5);
   for (uint32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < n; j += warps) {
-    const uint32_t pair = P.rows[j].x;
-    const int r = int(P.rows[j].y);
+    const uint32_t slot = P.scan[j], pair = P.span_list[P.spans[slot]];
     const Ell e = P.ell[pair];
+    const int r = int(slot - __float_as_uint(e.cx));
     const DevCam &cam = P.cams[pair / uint32_t(P.n)];
     const int ty = int(e.r0 >> 16) + r;
     int a = 0, b = -1;
     const bool any = scan_tile_span(P.rec[pair], cam, P.tile_w, float(ty * P.tile_h) + 0.5f,
                                     float(min((ty + 1) * P.tile_h, cam.H)) - 0.5f, int(e.r0 & 0xFFFF),
                                     int(e.r1 & 0xFFFF), a, b);
-    if ((threadIdx.x & 31) == 0)
-      P.spans[__float_as_uint(e.cx) + r] = any ? uint32_t(a) | (uint32_t(b - a + 1) << 16) : 0u;
+    if ((threadIdx.x & 31) == 0) P.spans[slot] = any ? uint32_t(a) | (uint32_t(b - a + 1) << 16) : 0u;
   }
 }
 
@@ -605,9 +607,11 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
           }
         } else if (i < n_inst) {
           // not a bounded ellipse: the span that pair_count_kernel computed, or the whole
-          // rectangle row (exact anti-aliasing bounds; no room left among the spans)
-          const uint32_t sb = A.z == -2.f ? kCulled : __float_as_uint(A.x);
-          const uint32_t sp = sb == kCulled ? tx0 | ((tx1 - tx0 + 1) << 16) : P.spans[sb + (i - C.x)];
+          // rectangle row (exact anti-aliasing bounds).  With more such rows than the capacity none
+          // of them has a span: which ones found room is not the same from call to call
+          const uint32_t sb = __float_as_uint(A.x);
+          const uint32_t sp = A.z == -2.f ? tx0 | ((tx1 - tx0 + 1) << 16)
+                              : P.counters->n_span_rows <= cap && sb != kCulled ? P.spans[sb + (i - C.x)] : 0u;
           xa_t = sp & 0xFFFFu;
           len = sp >> 16;
         }
