@@ -462,14 +462,12 @@ def run_ours(args, world, rank, local):
     peak_tf = sms * 128 * 2 * pk["sm_max_mhz"] * 1e6 / 1e12
     ach_tf = flops / (stages["render_ms"] * 1e-3) / 1e12
     # HBM view of the vertex stage: attributes read once; per visible pair the 64-B record,
-    # 8-B tile rectangle, 1-B tile-row count and 32-B support sector written; the 4-B key of
+    # 8-B tile rectangle, 2 B of tile rows and 32-B support sector written; the 4-B key of
     # every pair
     attr_bytes = sum(v.numel() * v.element_size() for v in st.values() if hasattr(v, "numel"))
-    prep_bytes = attr_bytes + 4 * n * len(cams) + 105 * ctr["n_visible"]
-    bin_bytes = binning_bytes(ctr, n * len(cams))
-    # kernels per pass: preprocess (2), depth sort (4 passes x 3), split by view (3), support
-    # rows (4), instance lists (2), rasteriser (1)
-    gpu_launches = args.steps * (2 + 12 + (3 if len(cams) > 1 else 0) + 4 + 2 + 1)
+    prep_bytes = attr_bytes + 4 * n * len(cams) + 106 * ctr["n_visible"]
+    bin_bytes = binning_pass_bytes(ctr, n * len(cams), len(cams))
+    gpu_launches = args.steps * launches_per_pass(n * len(cams), len(cams), sms)
 
     line = dict(
         metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,
@@ -493,6 +491,7 @@ def run_ours(args, world, rank, local):
         stages=dict(stages, preprocess_hbm_gbs=prep_bytes / (stages["preprocess_ms"] * 1e-3) / 1e9,
                     preprocess_hbm_frac=prep_bytes / (stages["preprocess_ms"] * 1e-3) / 1e9 / pk["hbm_gbs"],
                     bin_sort_bytes=bin_bytes,
+                    bin_sort_yardstick_bytes=binning_bytes(ctr, n * len(cams)),
                     bin_sort_hbm_gbs=bin_bytes / (stages["bin_sort_ms"] * 1e-3) / 1e9,
                     bin_sort_hbm_frac=bin_bytes / (stages["bin_sort_ms"] * 1e-3) / 1e9 / pk["hbm_gbs"]),
         autotune=tuned,
@@ -825,12 +824,42 @@ def precision_ablation(args, dev):
     return out
 
 
+SORT_ONE_CTA = 6144   # pairs up to which one CTA does the whole depth sort
+SORT_TILE = 2048      # items per CTA and step of a sort pass
+SORT_NO_SCAN = 16     # CTAs up to which a pass needs no scan kernel
+
+
+def launches_per_pass(pairs, views, sms):
+    """Kernels of one forward pass: vertex stage (2), depth sort (4 passes), split by view, support rows
+    (4), instance lists (2), rasteriser (1)."""
+    ctas = min(max(1, -(-pairs // SORT_TILE)), min(1024, 4 * sms))
+    sort_pass = 3 if ctas > SORT_NO_SCAN else 2
+    return 2 + (1 if pairs <= SORT_ONE_CTA else 4 * sort_pass) + (sort_pass if views > 1 else 0) + 4 + 2 + 1
+
+
+def binning_pass_bytes(ctr, pairs, views):
+    """Bytes that the kernels of a binning pass have to move, each array read or written once per use.
+    Depth sort: the dense 4-B keys (read twice, once by the upsweep), 2 B of tile rows per visible
+    pair and 8 B written, then per pass 4 B for the upsweep and 8 B in and out per pair (in one CTA:
+    no upsweeps, the passes between stay on chip).  Split by view: 4 + 8 B read, 12 B written.  Support
+    rows: 4 B of tile rows counted, then 8 B (12 B with several views) and the 32-B support
+    sector per pair, 8 B written per row.  Lists: the 8-B rows read twice, 4 B written per instance."""
+    nv, nr, ni = (int(ctr[k]) for k in ("n_visible", "n_rows", "n_instances"))
+    if pairs <= SORT_ONE_CTA:
+        depth = 4 * pairs + 2 * nv + 8 * nv
+    else:
+        depth = 8 * pairs + 2 * nv + 8 * nv + 3 * 20 * nv
+    split = 24 * nv if views > 1 else 0
+    rows = 4 * nv + (12 if views > 1 else 8) * nv + 32 * nv + 8 * nr
+    return depth + split + rows + 16 * nr + 4 * ni
+
+
 def binning_bytes(ctr, pairs):
-    """Algorithmic bytes of a binning pass that sorts the support rows by tile row in two passes
-    (each array read or written once per use; the row payload as stored), the yardstick of the
-    rates since the first version; the rows are now placed without that sort, so the bytes
-    really needed are fewer by row_sort less 8 B per kept row.  Depth sort (the dense 4-B keys and 1-B tile-row counts read,
-    then 8 B per visible pair per pass in and out, the upsweeps' key reads),
+    """Not what the kernels move: the algorithmic bytes of a binning pass that sorts the support rows by
+    tile row in two passes, as an earlier version did (each array read or written once per use; the
+    row payload as stored).  Kept as a yardstick of work, so that times of all versions can be
+    compared (binning_pass_bytes has the bytes of the present kernels).  Depth sort (the dense 4-B keys
+    and 1-B tile-row counts read, then 8 B per visible pair per pass in and out, the upsweeps' key reads),
     support rows (the 32-B support sector per pair, 12 B written per row), the tile-row
     sort (4-B key + 8-B payload read per row in the first pass, 12 B written per kept row,
     24 B per kept row in the second pass, the upsweeps' key reads), the chunk counts (the
