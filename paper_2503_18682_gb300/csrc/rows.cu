@@ -303,12 +303,12 @@ __device__ __forceinline__ void unbounded_spans(const PlaceParams &P) {
       int a0 = 0, b0 = -1, state = 0;
       if (r < rows) state = support_tile_span(rec, cam, P.tile_w, ya, yb, tx0, tx1, a0, b0);
       uint32_t span = state ? uint32_t(a0) | (uint32_t(b0 - a0 + 1) << 16) : 0u;
-      if (state < 0) {  // left to scan_rows; until then the span holds the pair's place in the list
+      if (state < 0) {  // left to scan_rows; until then the span holds the pair
         span = uint32_t(tx0) | (uint32_t(tx1 - tx0 + 1) << 16);
         const uint32_t j = atomicAdd(&P.counters->n_scan, 1u);
         if (j < P.cap) {  // (always: there are no more spans)
           P.scan[j] = base + uint32_t(r);
-          span = uint32_t(u / parts);
+          span = pair;
         }
       }
       if (r < rows) P.spans[base + r] = span;
@@ -320,8 +320,14 @@ __device__ __forceinline__ void unbounded_spans(const PlaceParams &P) {
 __device__ __forceinline__ void scan_rows(const PlaceParams &P) {
   const uint32_t n = min(P.counters->n_scan, P.cap);
   const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-  for (uint32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < n; j += warps) {
-    const uint32_t slot = P.scan[j], pair = P.span_list[P.spans[slot]];
+  uint32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  uint32_t next_slot = j < n ? P.scan[j] : 0u, next_pair = j < n ? P.spans[next_slot] : 0u;
+  for (; j < n; j += warps) {
+    const uint32_t slot = next_slot, pair = next_pair;
+    if (j + warps < n) {  // (a span is read and then written by the one warp that tests its row)
+      next_slot = P.scan[j + warps];
+      next_pair = P.spans[next_slot];
+    }
     const Ell e = P.ell[pair];
     const int r = int(slot - __float_as_uint(e.cx));
     const DevCam &cam = P.cams[pair / uint32_t(P.n)];
@@ -528,6 +534,9 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
   for (int i = lane; i < W; i += 32) tog[i] = 0u;
   build_view_tab(P, T);
   const uint32_t nchunks = T.chunk0[P.n_views], cap = P.cap;
+  // With more rows of unbounded supports than the capacity none of them has a span: which ones found room
+  // is not the same from call to call.
+  const uint32_t span_end = P.counters->n_span_rows <= cap ? cap : 0u;
   uint32_t kept = 0;
   for (uint32_t c = blockIdx.x * NW + warp; c < nchunks; c += gridDim.x * NW) {
     const Chunk ck = chunk_at(T, P.n_views, c);
@@ -607,11 +616,9 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
           }
         } else if (i < n_inst) {
           // not a bounded ellipse: the span that pair_count_kernel computed, or the whole
-          // rectangle row (exact anti-aliasing bounds).  With more such rows than the capacity none
-          // of them has a span: which ones found room is not the same from call to call
+          // rectangle row (exact anti-aliasing bounds)
           const uint32_t sb = __float_as_uint(A.x);
-          const uint32_t sp = A.z == -2.f ? tx0 | ((tx1 - tx0 + 1) << 16)
-                              : P.counters->n_span_rows <= cap && sb != kCulled ? P.spans[sb + (i - C.x)] : 0u;
+          const uint32_t sp = A.z == -2.f ? tx0 | ((tx1 - tx0 + 1) << 16) : sb < span_end ? P.spans[sb + (i - C.x)] : 0u;
           xa_t = sp & 0xFFFFu;
           len = sp >> 16;
         }
