@@ -288,10 +288,11 @@ static size_t list_smem(int max_tiles_x) {
 // counts of all the tile row's chunks), short ones still occupy every SM.  A 720p frame's 0.43 M
 // rows in chunks of 512: 17 us, against 39 us in chunks of 8,192 (90 of them).  Longer when the
 // per-chunk column counts would pass 32 M entries.
-// On views wider than 512 tiles the shortest chunk has a row per tile column at least: the column
-// counts then take no more than 4 bytes per unit of capacity.
-uint32_t list_rows_lo(int max_tiles_x) {
-  uint32_t cr = 512;
+// With a shortest chunk of a row per tile column at least, the column counts take no more than 4 bytes
+// per unit of capacity, on views wider than 512 tiles too (at 512 rows up to 32 bytes): where the
+// workspace is short.  It costs time there (32768x512, 50k primitives: binning 147 against 128 us).
+uint32_t list_rows_short(int max_tiles_x) {
+  uint32_t cr = kListRowsLo;
   while (cr < uint32_t(max_tiles_x)) cr <<= 1;
   return cr;
 }
@@ -301,8 +302,8 @@ uint32_t list_rows_hi(int64_t cap, int max_tiles_x) {
   return cr;
 }
 uint32_t list_target(int num_sms) { return uint32_t(num_sms) * 16; }
-uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sms) {
-  const uint64_t by_lo = uint64_t(cap) / list_rows_lo(max_tiles_x), by_hi = uint64_t(cap) / list_rows_hi(cap, max_tiles_x);
+uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sms, uint32_t rows_lo) {
+  const uint64_t by_lo = uint64_t(cap) / rows_lo, by_hi = uint64_t(cap) / list_rows_hi(cap, max_tiles_x);
   return uint64_t(trows) + std::min<uint64_t>(by_lo, std::max<uint64_t>(list_target(num_sms), by_hi)) + 1;
 }
 

@@ -42,38 +42,39 @@ raygs_status scratch_for_current_device(void **out) {
 }
 
 // Size check: the fixed part must fit; the rest of the array bounds the tile rows and instances.  What only
-// makes a pass faster (the row pass's head chunks, the tiles by class on small batches) is left
-// out of a batch that would otherwise not fit, or keep less than half of the capacity.
+// makes a pass faster (the row pass's head chunks, the tiles by class on small batches, short chunks of
+// wide views in the list pass) is left out of a batch that would otherwise not fit, or keep less than two
+// thirds of the capacity.
 bool fit_scratch(Work &w) {
-  const struct { int heads; bool order; } keep[] = {{kHeadChunks, w.tiles <= 8192}, {16, false}, {0, false}};
-  Work best[3];
-  for (int i = 2; i >= 0; --i) {
-    Work &c = best[i];
-    c = w;
-    LayoutOptions opt;
-    opt.tile_stop = false;
-    opt.bin_once = true;
+  const uint32_t rows_short = list_rows_short(w.max_tiles_x);
+  const struct { int heads; bool order; uint32_t list_lo; } keep[] = {
+      {kHeadChunks, w.tiles <= 8192, kListRowsLo}, {16, false, rows_short}, {0, false, rows_short}};
+  LayoutOptions opt;
+  opt.tile_stop = false;
+  opt.bin_once = true;
+  int64_t most = 0;  // what the barest layout leaves
+  for (int i : {2, 0, 1, 2}) {
     opt.tile_order = keep[i].order;
-    opt.heads = c.heads = keep[i].heads;
+    opt.heads = w.heads = keep[i].heads;
+    opt.list_lo = w.list_lo = keep[i].list_lo;
     auto layout = [&](int64_t cap) {
-      c.cap = cap;
-      c.L = make_layout(c.n_views, c.n, c.tiles, c.trows, cap, c.num_sms, c.max_tiles_x, c.max_rows, opt);
-      return c.L.total <= kNoAllocScratchBytes;
+      w.cap = cap;
+      w.L = make_layout(w.n_views, w.n, w.tiles, w.trows, cap, w.num_sms, w.max_tiles_x, w.max_rows, opt);
+      return w.L.total <= kNoAllocScratchBytes;
     };
     layout(0);
-    const double room = double(kNoAllocScratchBytes) - double(c.L.total);
+    const double room = double(kNoAllocScratchBytes) - double(w.L.total);
     // the column counts: up to so many bytes per unit of capacity, and no more than so many in all
-    const double per_unit = 4.0 * c.max_tiles_x / list_rows_lo(c.max_tiles_x);
-    const double in_all = 4.0 * c.max_tiles_x * list_target(c.num_sms);
+    const double per_unit = 4.0 * w.max_tiles_x / w.list_lo, in_all = 4.0 * w.max_tiles_x * list_target(w.num_sms);
     int64_t cap = int64_t(std::max(room / (kBytesPerCapacity + per_unit), (room - in_all) / kBytesPerCapacity));
-    while (cap > 0 && !layout(cap)) cap -= 256;
-    if (cap <= 0) c.cap = 0;
-  }
-  for (const Work &c : best)
-    if (c.cap > 0 && 2 * c.cap >= best[2].cap) {
-      w = c;
-      return true;
+    if (most == 0) {
+      if (cap <= 0) return false;
+      most = cap;
+      continue;
     }
+    while (cap > 0 && !layout(cap)) cap -= 256;
+    if (cap > 0 && (3 * cap >= 2 * most || i == 2)) return true;
+  }
   return false;
 }
 

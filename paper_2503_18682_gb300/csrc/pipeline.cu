@@ -107,7 +107,7 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.trange = take(8 * size_t(trows) + 16);
   L.trinst = take(8 * size_t(trows) + 16);
   L.cbase = take(4 * size_t(trows + 1) + 16);
-  L.ccnt = take(4 * size_t(list_max_chunks(trows, cap, max_tiles_x, num_sms)) * size_t(max_tiles_x) + 16);
+  L.ccnt = take(4 * size_t(list_max_chunks(trows, cap, max_tiles_x, num_sms, opt.list_lo)) * size_t(max_tiles_x) + 16);
   L.hist = take(4 * 256 * size_t(sort_blocks(VN, sort_grid(num_sms))));
   L.dtot = take(4 * 256);
   L.ranges = take(8 * size_t(tiles));
@@ -271,10 +271,10 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   R.trow_inst = w.at<unsigned long long>(w.L.trinst);
   R.rows = w.at<uint2>(w.L.rows);
   R.chunk_base = w.at<uint32_t>(w.L.cbase);
-  R.list_lo = list_rows_lo(w.max_tiles_x);
+  R.list_lo = w.list_lo;
   R.list_hi = list_rows_hi(w.cap, w.max_tiles_x);
   R.list_target = list_target(w.num_sms);
-  R.max_chunks = uint32_t(list_max_chunks(w.trows, w.cap, w.max_tiles_x, w.num_sms));
+  R.max_chunks = uint32_t(list_max_chunks(w.trows, w.cap, w.max_tiles_x, w.num_sms, w.list_lo));
   const bool backward = w.cfg.enable_backward != 0;
   R.row_e = backward ? w.at<uint2>(w.L.re) : nullptr;
   R.e_base = backward ? w.at<uint32_t>(w.L.ebase) : nullptr;

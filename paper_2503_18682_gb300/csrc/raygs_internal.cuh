@@ -400,10 +400,11 @@ constexpr int kHeadChunks = 128;  // head chunks of a view in the row pass, wher
 uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows, int heads);
 uint64_t place_max_counts(int n_views, uint64_t pairs, int max_rows, int64_t trows, int heads);
 cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st);
-uint32_t list_rows_lo(int max_tiles_x);
+constexpr uint32_t kListRowsLo = 512;  // rows of the shortest chunk of the list pass
+uint32_t list_rows_short(int max_tiles_x);
 uint32_t list_rows_hi(int64_t cap, int max_tiles_x);
 uint32_t list_target(int num_sms);
-uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sms);
+uint64_t list_max_chunks(int64_t trows, int64_t cap, int max_tiles_x, int num_sms, uint32_t rows_lo);
 cudaError_t launch_lists(const ListParams &P, int num_sms, cudaStream_t st);
 cudaError_t launch_render(const RenderParams &P, int tile_w, int tile_h, int batch_records, int num_sms,
                           bool count, cudaStream_t st);
@@ -429,6 +430,7 @@ struct LayoutOptions {
   bool tile_stop = true;    // per-tile stop positions (instrumented renders)
   bool bin_once = false;    // one binning per vertex stage: what it reads of that need not outlast it
   int heads = kHeadChunks;  // head chunks of a view in the row pass (their counts: 4 bytes per tile row each)
+  uint32_t list_lo = kListRowsLo;  // rows of the shortest chunk of the list pass (its counts: 4 bytes per tile column)
 };
 
 Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t cap, int num_sms, int max_tiles_x,
@@ -450,6 +452,7 @@ struct Work {
   int64_t n = 0, tiles = 0, trows = 0, cap = 0;
   int max_tiles_x = 0, max_rows = 0;  // most tile columns and rows of one view
   int G = 0, num_sms = 0, heads = kHeadChunks;
+  uint32_t list_lo = kListRowsLo;
   raygs_config cfg{};
   int s1_final = 0;  // which ping-pong buffer holds the depth-sorted pairs
   template <typename T>
