@@ -42,8 +42,8 @@ __device__ __forceinline__ uint32_t pass_count(const SortPass &p) {
 }
 
 // Digit histogram of the CTA's items.  Each thread counts 16 consecutive keys as runs of
-// equal digits (the tile-id passes see long runs: instances come in depth order, tile rows
-// in order) and adds each run once to its warp's shared histogram.
+// equal digits (the top digit of a depth is little more than its exponent, and the views are few:
+// long runs) and adds each run once to its warp's shared histogram.
 template <int BITS, bool FILTER>
 __global__ void __launch_bounds__(kSortThreads) sort_upsweep(SortPass p) {
   await_previous();
@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(kSortThreads) sort_upsweep(SortPass p) {
 
 // MODE: what a pass does with its payloads.  First drops the culled keys and packs the tile
 // rows beside key and id, last unpacks them (see SortPass), split also writes the items'
-// indices; compiled apart, so that the plain passes keep their 64 registers.
+// indices; compiled apart, so that the plain passes keep their 64 registers (the first and
+// the last pass spill 16 bytes at that bound, the split by up to 16 views 68, by more 48).
 enum SortMode { kSortPlain = 0, kSortFirst = 1, kSortLast = 2, kSortSplit = 3 };
 
 template <int BITS, int MODE>
