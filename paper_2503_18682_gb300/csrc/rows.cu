@@ -201,12 +201,16 @@ struct ViewTab {
   uint32_t head0[RAYGS_MAX_VIEWS + 1];   // head chunks of the views before it
   uint32_t entry0[RAYGS_MAX_VIEWS + 1];  // its first count (tile rows x chunks)
   uint32_t cp;
+  // End of the spans of unbounded supports.  With more of their rows than the capacity none of them has a span:
+  // which ones found room is not the same from call to call.
+  uint32_t span_end;
 };
 
 __device__ __forceinline__ void build_view_tab(const PlaceParams &P, ViewTab &T) {
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     const uint32_t nvis = P.counters->n_visible;
+    const unsigned long long span_rows = P.counters->n_span_rows;
     uint32_t cp = P.cp_lo;
     while (cp < P.cp_hi && nvis / cp >= P.target) cp <<= 1;
     uint32_t s0 = 0, c0 = 0, h0 = 0, e0 = 0;
@@ -235,6 +239,7 @@ __device__ __forceinline__ void build_view_tab(const PlaceParams &P, ViewTab &T)
       T.head0[P.n_views] = h0;
       T.entry0[P.n_views] = e0;
       T.cp = cp;
+      T.span_end = span_rows <= P.cap ? P.cap : 0u;
     }
   }
   __syncthreads();
@@ -534,9 +539,6 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
   for (int i = lane; i < W; i += 32) tog[i] = 0u;
   build_view_tab(P, T);
   const uint32_t nchunks = T.chunk0[P.n_views], cap = P.cap;
-  // With more rows of unbounded supports than the capacity none of them has a span: which ones found room
-  // is not the same from call to call.
-  const uint32_t span_end = P.counters->n_span_rows <= cap ? cap : 0u;
   uint32_t kept = 0;
   for (uint32_t c = blockIdx.x * NW + warp; c < nchunks; c += gridDim.x * NW) {
     const Chunk ck = chunk_at(T, P.n_views, c);
@@ -618,7 +620,7 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
           // not a bounded ellipse: the span that pair_count_kernel computed, or the whole
           // rectangle row (exact anti-aliasing bounds)
           const uint32_t sb = __float_as_uint(A.x);
-          const uint32_t sp = A.z == -2.f ? tx0 | ((tx1 - tx0 + 1) << 16) : sb < span_end ? P.spans[sb + (i - C.x)] : 0u;
+          const uint32_t sp = A.z == -2.f ? tx0 | ((tx1 - tx0 + 1) << 16) : sb < T.span_end ? P.spans[sb + (i - C.x)] : 0u;
           xa_t = sp & 0xFFFFu;
           len = sp >> 16;
         }
