@@ -169,6 +169,8 @@ __global__ void __launch_bounds__(NT) list_kernel(ListParams P) {
   uint32_t *s_cur = s_mem;                   // [TX] next free slot of each tile
   uint32_t *s_pre = s_cur + TX;              // [VW][TP] first slot of each group
   uint32_t *s_mask = s_pre + VW * TP;        // [2][VW][TP]
+  __shared__ uint32_t s_longest;             // longest of the tile row's lists (chunk 0)
+  if (threadIdx.x == 0) s_longest = 0u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t tile0 = uint32_t(cam.tile_base) + uint32_t(grow - cam.trow_base) * uint32_t(TX);
@@ -195,7 +197,7 @@ __global__ void __launch_bounds__(NT) list_kernel(ListParams P) {
     uint32_t ctot;
     const uint32_t cpre = block_excl_scan(csum, s_ws, &ctot);  // instances before the column chunk
     const unsigned long long base = P.trow_inst[grow];
-    uint32_t o = uint32_t(min(base, (unsigned long long)P.cap)) + cpre;
+    uint32_t o = uint32_t(min(base, (unsigned long long)P.cap)) + cpre, longest = 0;
     for (int x = x0; x < x1; ++x) {
       const uint32_t n = s_tot[x];
       s_cur[x] = o + s_bef[x];
@@ -203,14 +205,18 @@ __global__ void __launch_bounds__(NT) list_kernel(ListParams P) {
         const uint2 r = make_uint2(min(o, P.cap), min(o + n, P.cap));
         P.ranges[tile0 + x] = r;
         if (P.class_tiles) {
+          longest = max(longest, r.y - r.x);
           const int c = tile_class_of(r.y - r.x);
           P.class_tiles[size_t(c) * size_t(P.tiles) + atomicAdd(&P.counters->tile_class[c], 1u)] = tile0 + x;
         }
       }
       o += n;
     }
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    if (lane == 0 && longest) atomicMax(&s_longest, longest);
   }
   __syncthreads();
+  if (threadIdx.x == 0 && s_longest) atomicMax(&P.counters->longest, s_longest);
   for (int j = threadIdx.x; j < 2 * VW * TP; j += NT) s_mask[j] = 0u;
   constexpr uint32_t STEP = uint32_t(NT) * KR;
   uint2 nxt[KR];

@@ -331,7 +331,8 @@ cudaError_t run_render(const Work &w, float *rgb, float *T_final, int32_t *n_con
   P.tile_counter = w.at<unsigned int>(w.L.tilectr);
   P.n_tiles = int(w.tiles);
   P.class_tiles = w.L.tclass ? w.at<uint32_t>(w.L.tclass) : nullptr;
-  P.class_count = w.at<Counters>(w.L.counters)->tile_class;
+  P.counters = w.at<Counters>(w.L.counters);
+  P.class_count = P.counters->tile_class;
   if (P.recx) return launch_render_mipx(P, w.cfg.tile_w, w.cfg.tile_h, w.num_sms, count, st);
   return launch_render(P, w.cfg.tile_w, w.cfg.tile_h, w.cfg.batch_records, w.num_sms, count, st);
 }

@@ -58,6 +58,7 @@ struct Counters {
   uint32_t n_scan;          // rows of those pairs that have to be tested tile by tile
   uint32_t chunk_rows;      // rows per chunk of the list pass
   uint32_t lists_done;      // CTAs of list_count_kernel that have finished (0 between launches)
+  uint32_t longest;                           // longest list of a tile (0 where no classes are kept)
   uint32_t tile_class[16];                    // tiles of each class (see tile_class_of)
 };
 
@@ -282,6 +283,7 @@ struct RenderParams {
   int n_tiles;
   const uint32_t *class_tiles;  // tiles by class (nullable: tile order)
   const uint32_t *class_count;
+  const Counters *counters;
   int slots;                    // CTAs resident at a time (set at the launch)
   const Rec *recx;  // exact anti-aliasing: second half of each record (then rec holds the first)
   float p_min;

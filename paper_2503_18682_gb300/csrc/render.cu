@@ -255,6 +255,12 @@ __global__ void __launch_bounds__(TW *TH / PX, 16) render_kernel(RenderParams P)
 // the whole-tile kernel, bit for bit.  720p, 500k primitives: 131 us against 179 in whole tiles
 // (151 with one pixel per thread), 1.5M: 174 against 217 (212); four uneven 640x480 views of 200k:
 // 77 us with one pixel per thread, 117 with two, 191 in whole tiles; 64x64, 1k: 19, 29 and 48.
+// Where the lists are even enough that the longest one does not set the time (large primitives, a camera
+// inside them, an empty view), the most pixels per thread and no lists of the warps: 100k large
+// primitives at 1280x720 117 us against 133 in parts, 5k around the camera 56 against 77, an empty
+// 1600x900 view 17 against 25 (16x8 tiles 117 against 137, 60 against 76; 32x16 tiles, then in halves, 126
+// against 141, 61 against 83).  The line at 0.4 of the longest list per slot: 100k middling primitives at
+// 960x540 (0.34) 79 us in parts against 77, at 1280x720 (0.6) 116 against 111.
 template <int TW, int TH, int NBF, int DIV>
 __global__ void __launch_bounds__(64, 18) render_parts_kernel(RenderParams P) {
   await_previous();
@@ -264,7 +270,11 @@ __global__ void __launch_bounds__(64, 18) render_parts_kernel(RenderParams P) {
   // tiles with 64 records and more (class 9 is the last of them)
   static_assert(tile_class_min(9) == 64, "classes");
   const bool fine = P.class_tiles && M.items.first[10] * uint32_t((TW / 8) * (TH / 8)) <= uint32_t(P.slots);
-  if (PX == 1 || fine) render_regions<TW, TH, 8, 8, 1, NBF, true, false, DIV>(P, M);
+  // the lists' sum per slot at least 0.4 of the longest one, in lists of 16x16 tiles
+  const uint2 lists = M.items.lists;
+  const bool even = P.class_tiles && 10ull * TW * TH * lists.x >= 4ull * 256 * uint32_t(P.slots) * lists.y;
+  if (TW >= 16 && even) render_regions<TW, TH, 16, TH, TH / 4, NBF, false, false, DIV>(P, M);
+  else if (PX == 1 || fine) render_regions<TW, TH, 8, 8, 1, NBF, true, false, DIV>(P, M);
   else render_regions<TW, TH, RW, RH, PX, NBF, true, false, DIV>(P, M);
   leave_items(P);
 }

@@ -491,6 +491,7 @@ __global__ void __launch_bounds__(1024) trow_plan_kernel(PlaceParams P) {
     P.counters->n_rows_clamped = uint32_t(min(tot, cap));
     P.counters->n_rows_kept = 0u;
     P.counters->n_scan = 0u;
+    P.counters->longest = 0u;
     for (int c = 0; c < kTileClasses; ++c) P.counters->tile_class[c] = 0u;
     P.counters->n_partials = 0u;
     if (tot > cap) P.counters->overflow = 1u;
