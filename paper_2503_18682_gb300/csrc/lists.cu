@@ -198,16 +198,22 @@ __global__ void __launch_bounds__(NT) list_kernel(ListParams P) {
     const uint32_t cpre = block_excl_scan(csum, s_ws, &ctot);  // instances before the column chunk
     const unsigned long long base = P.trow_inst[grow];
     uint32_t o = uint32_t(min(base, (unsigned long long)P.cap)) + cpre, longest = 0;
-    for (int x = x0; x < x1; ++x) {
-      const uint32_t n = s_tot[x];
-      s_cur[x] = o + s_bef[x];
+    for (int j = 0; j < per; ++j) {
+      const int x = x0 + j;
+      const bool in = x < x1;
+      const uint32_t n = in ? s_tot[x] : 0u;
+      if (in) s_cur[x] = o + s_bef[x];
       if (chunk_c == 0) {
         const uint2 r = make_uint2(min(o, P.cap), min(o + n, P.cap));
-        P.ranges[tile0 + x] = r;
-        if (P.class_tiles) {
+        if (in) P.ranges[tile0 + x] = r;
+        if (P.class_tiles) {  // one atomic per class and warp: of 518,400 tiles one by one they took 260 us
           longest = max(longest, r.y - r.x);
-          const int c = tile_class_of(r.y - r.x);
-          P.class_tiles[size_t(c) * size_t(P.tiles) + atomicAdd(&P.counters->tile_class[c], 1u)] = tile0 + x;
+          const int c = in ? tile_class_of(r.y - r.x) : kTileClasses;
+          const uint32_t peers = __match_any_sync(0xffffffffu, c);
+          uint32_t at = 0;
+          if (in && lane == __ffs(peers) - 1) at = atomicAdd(&P.counters->tile_class[c], __popc(peers));
+          at = __shfl_sync(0xffffffffu, at, __ffs(peers) - 1) + __popc(peers & lt);
+          if (in) P.class_tiles[size_t(c) * size_t(P.tiles) + at] = tile0 + x;
         }
       }
       o += n;
