@@ -8,8 +8,8 @@
 // lane.  Two shared-memory atomics per item, whatever it covers, and no barrier beyond the
 // warp.  The instances of the 32 items are then taken 32 at a time, one per lane.
 //
-// Lane l owns the bins [l nj, (l + 1) nj), nj odd (no bank conflicts); with J > 0 nj = J and
-// the cursors live in registers, with J = 0 nj is a run-time value and they stay in the table.
+// Lane l owns the bins [l J, (l + 1) J), J odd (no bank conflicts), their cursors in registers.  The counts
+// work for a run-time number of bins per lane too (J = 0).
 #pragma once
 
 #include "raygs_internal.cuh"
@@ -69,19 +69,14 @@ __device__ __forceinline__ void bins_counts(uint32_t *diff, uint32_t *cnt, int n
 // Masks of 32 items from their toggles: mc[b] = (lanes covering b, cursor of b before these
 // items); the cursors advance past them and the toggles are cleared.
 template <int J>
-__device__ __forceinline__ void bins_masks(uint32_t *tog, uint2 *mc, int nj_dyn, uint32_t (&cur)[J ? J : 1]) {
-  const int lane = threadIdx.x & 31;
-  const int nj = J ? J : nj_dyn, b0 = lane * nj;
-  uint32_t loc[J ? J : 1], x = 0;
-  if (J) {
+__device__ __forceinline__ void bins_masks(uint32_t *tog, uint2 *mc, uint32_t (&cur)[J]) {
+  const int lane = threadIdx.x & 31, b0 = lane * J;
+  uint32_t loc[J], x = 0;
 #pragma unroll
-    for (int j = 0; j < (J ? J : 1); ++j) {
-      x ^= tog[b0 + j];
-      tog[b0 + j] = 0u;
-      loc[j] = x;
-    }
-  } else {
-    for (int j = 0; j < nj; ++j) x ^= tog[b0 + j];
+  for (int j = 0; j < J; ++j) {
+    x ^= tog[b0 + j];
+    tog[b0 + j] = 0u;
+    loc[j] = x;
   }
   uint32_t s = x;
 #pragma unroll
@@ -89,21 +84,12 @@ __device__ __forceinline__ void bins_masks(uint32_t *tog, uint2 *mc, int nj_dyn,
     const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
     if (lane >= o) s ^= y;
   }
-  uint32_t carry = s ^ x;  // toggles of the lower lanes' bins
-  if (J) {
+  const uint32_t carry = s ^ x;  // toggles of the lower lanes' bins
 #pragma unroll
-    for (int j = 0; j < (J ? J : 1); ++j) {
-      const uint32_t m = loc[j] ^ carry;
-      mc[b0 + j] = make_uint2(m, cur[j]);
-      cur[j] += __popc(m);
-    }
-  } else {
-    for (int j = 0; j < nj; ++j) {
-      carry ^= tog[b0 + j];
-      tog[b0 + j] = 0u;
-      const uint2 o = mc[b0 + j];
-      mc[b0 + j] = make_uint2(carry, o.y + __popc(o.x));
-    }
+  for (int j = 0; j < J; ++j) {
+    const uint32_t m = loc[j] ^ carry;
+    mc[b0 + j] = make_uint2(m, cur[j]);
+    cur[j] += __popc(m);
   }
   __syncwarp();
 }

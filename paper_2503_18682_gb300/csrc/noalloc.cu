@@ -52,6 +52,7 @@ bool fit_scratch(Work &w) {
   LayoutOptions opt;
   opt.tile_stop = false;
   opt.bin_once = true;
+  opt.short_chunks = w.short_chunks = false;
   int64_t most = 0;  // what the barest layout leaves
   for (int i : {2, 0, 1, 2}) {
     opt.tile_order = keep[i].order;

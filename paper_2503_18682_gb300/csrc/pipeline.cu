@@ -93,8 +93,10 @@ Layout make_layout(int n_views, int64_t n, int64_t tiles, int64_t trows, int64_t
   L.recx = opt.mip_exact ? take(sizeof(Rec) * VN) : 0;
   for (int i = 0; i < 2; ++i) { L.s1k[i] = take(4 * VN); L.s1v[i] = take(4 * VN); }
   L.vpos = n_views > 1 ? take(4 * VN) : 0;
-  const uint64_t pchunks = place_max_chunks(n_views, VN, max_rows, opt.heads);
-  L.cnt1 = take(4 * size_t(place_max_counts(n_views, VN, max_rows, trows, opt.heads)) + 16);
+  const uint32_t chunk_lo = place_chunk_lo(VN, max_rows, opt.short_chunks);
+  const int heads = opt.heads < 0 ? place_heads(max_rows, trows, opt.short_chunks) : opt.heads;
+  const uint64_t pchunks = place_max_chunks(n_views, VN, chunk_lo, heads);
+  L.cnt1 = take(4 * size_t(place_max_counts(n_views, VN, max_rows, trows, chunk_lo, heads)) + 16);
   // per unit of capacity: kBytesPerCapacity bytes
   L.rows = take(8 * C + 16);
   L.spanl = opt.bin_once ? L.rows + 4 * C : take(4 * size_t(span_list_cap(VN, C)));
@@ -261,7 +263,8 @@ cudaError_t run_bin_sort(Work &w, cudaStream_t st) {
   R.trows = int(w.trows);
   R.max_rows = w.max_rows;
   R.cap = cap;
-  R.heads = uint32_t(w.heads);
+  R.heads = uint32_t(w.heads < 0 ? place_heads(w.max_rows, w.trows, w.short_chunks) : w.heads);
+  R.cp_lo = place_chunk_lo(VN, w.max_rows, w.short_chunks);
   R.span_list = w.at<uint32_t>(w.L.spanl);
   R.span_list_cap = span_list_cap(VN, cap);
   R.spans = w.at<uint32_t>(w.L.spans);

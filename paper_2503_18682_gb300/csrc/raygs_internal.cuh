@@ -224,7 +224,7 @@ struct PlaceParams {
   int n, n_views, tile_w, tile_h;
   int trows, max_rows;         // tile rows of the batch, and the most of one view
   uint32_t cap;
-  uint32_t heads;              // head chunks of a view, at most (see rows.cu)
+  uint32_t heads, head_pairs;  // head chunks of a view, at most, and their pairs (see rows.cu)
   uint32_t cp_lo, cp_hi, target;
   const uint32_t *span_list;   // pairs whose support is not a bounded ellipse (see PrepParams)
   uint32_t span_list_cap;
@@ -399,8 +399,11 @@ bool sort_is_small(uint64_t pairs);  // one kernel for the whole depth sort
 cudaError_t launch_sort_small(const SortPass &p, cudaStream_t st);  // row_info, row_rect and d_total set
 int sort_blocks(uint64_t items, int grid);  // CTAs of a pass
 constexpr int kHeadChunks = 128;  // head chunks of a view in the row pass, where there is room for their counts
-uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows, int heads);
-uint64_t place_max_counts(int n_views, uint64_t pairs, int max_rows, int64_t trows, int heads);
+uint32_t place_chunk_lo(uint64_t pairs, int max_rows, bool short_chunks);
+int place_heads(int max_rows, int64_t trows, bool short_chunks);
+uint32_t place_head_pairs(int heads);
+uint64_t place_max_chunks(int n_views, uint64_t pairs, uint32_t chunk_lo, int heads);
+uint64_t place_max_counts(int n_views, uint64_t pairs, int max_rows, int64_t trows, uint32_t chunk_lo, int heads);
 cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st);
 constexpr uint32_t kListRowsLo = 512;  // rows of the shortest chunk of the list pass
 uint32_t list_rows_short(int max_tiles_x);
@@ -431,7 +434,8 @@ struct LayoutOptions {
   bool tile_order = true;   // the tiles by class (48 bytes per tile): without, they are taken in tile order
   bool tile_stop = true;    // per-tile stop positions (instrumented renders)
   bool bin_once = false;    // one binning per vertex stage: what it reads of that need not outlast it
-  int heads = kHeadChunks;  // head chunks of a view in the row pass (their counts: 4 bytes per tile row each)
+  int heads = -1;           // head chunks of a view in the row pass (their counts: 4 bytes per tile row each); -1: place_heads
+  bool short_chunks = true;        // short chunks of the row pass on tall views (see place_chunk_lo)
   uint32_t list_lo = kListRowsLo;  // rows of the shortest chunk of the list pass (its counts: 4 bytes per tile column)
 };
 
@@ -453,7 +457,8 @@ struct Work {
   int n_views = 0;
   int64_t n = 0, tiles = 0, trows = 0, cap = 0;
   int max_tiles_x = 0, max_rows = 0;  // most tile columns and rows of one view
-  int G = 0, num_sms = 0, heads = kHeadChunks;
+  int G = 0, num_sms = 0, heads = -1;
+  bool short_chunks = true;
   uint32_t list_lo = kListRowsLo;
   raygs_config cfg{};
   int s1_final = 0;  // which ping-pong buffer holds the depth-sorted pairs

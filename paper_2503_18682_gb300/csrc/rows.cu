@@ -188,19 +188,18 @@ __device__ __noinline__ bool scan_tile_span(const Rec &r, const DevCam &cam, int
 
 // The views' shares of the sorted pairs and their chunks.  A view's nearest pairs are its
 // largest ones (up to all its tile rows each, where the average is three), so its first
-// P.heads chunks hold only kHeadPairs pairs, and the batch takes all views' head chunks
+// P.heads chunks hold only P.head_pairs pairs, and the batch takes all views' head chunks
 // first (kHeadChunks of them; fewer or none where the workspace has no room for their counts).
 //  The other chunks' length is the smallest power of two in [cp_lo, cp_hi] that leaves
 // no more than `target` chunks: short lists still give every SM work, long ones amortise a
 // chunk's scans and write longer runs.
-constexpr uint32_t kHeadPairs = 16;
 
 struct ViewTab {
   uint32_t start[RAYGS_MAX_VIEWS + 1];   // first sorted pair of the view
   uint32_t chunk0[RAYGS_MAX_VIEWS + 1];  // chunks of the views before it
   uint32_t head0[RAYGS_MAX_VIEWS + 1];   // head chunks of the views before it
   uint32_t entry0[RAYGS_MAX_VIEWS + 1];  // its first count (tile rows x chunks)
-  uint32_t cp;
+  uint32_t cp, head_pairs;
   // End of the spans of unbounded supports.  With more of their rows than the capacity none of them has a span:
   // which ones found room is not the same from call to call.
   uint32_t span_end;
@@ -218,8 +217,8 @@ __device__ __forceinline__ void build_view_tab(const PlaceParams &P, ViewTab &T)
       const int v = h + lane;
       const bool in = v < P.n_views;
       const uint32_t n = in ? (P.view_count ? P.view_count[v] : nvis) : 0u;
-      const uint32_t nh = min(P.heads, (n + kHeadPairs - 1) / kHeadPairs);
-      const uint32_t nch = nh + (n > nh * kHeadPairs ? (n - nh * kHeadPairs + cp - 1) / cp : 0u);
+      const uint32_t nh = min(P.heads, (n + P.head_pairs - 1) / P.head_pairs);
+      const uint32_t nch = nh + (n > nh * P.head_pairs ? (n - nh * P.head_pairs + cp - 1) / cp : 0u);
       const uint32_t e = in ? nch * uint32_t(P.cams[v].tiles_y) : 0u;
       const uint32_t si = warp_incl_scan(n), ci = warp_incl_scan(nch), hi = warp_incl_scan(nh), ei = warp_incl_scan(e);
       if (in) {
@@ -239,6 +238,7 @@ __device__ __forceinline__ void build_view_tab(const PlaceParams &P, ViewTab &T)
       T.head0[P.n_views] = h0;
       T.entry0[P.n_views] = e0;
       T.cp = cp;
+      T.head_pairs = P.head_pairs;
       T.span_end = span_rows <= P.cap ? P.cap : 0u;
     }
   }
@@ -266,9 +266,9 @@ __device__ __forceinline__ Chunk chunk_at(const ViewTab &T, int n_views, uint32_
   k.v = v;
   const uint32_t nh = T.head0[v + 1] - T.head0[v];
   k.nch = T.chunk0[v + 1] - T.chunk0[v];
-  k.cp = head ? kHeadPairs : T.cp;
+  k.cp = head ? T.head_pairs : T.cp;
   k.cc = head ? c - T.head0[v] : nh + c - (heads + T.chunk0[v] - T.head0[v]);
-  k.q0 = T.start[v] + (head ? k.cc * kHeadPairs : nh * kHeadPairs + (k.cc - nh) * T.cp);
+  k.q0 = T.start[v] + (head ? k.cc * T.head_pairs : nh * T.head_pairs + (k.cc - nh) * T.cp);
   k.q1 = min(k.q0 + k.cp, T.start[v + 1]);
   return k;
 }
@@ -519,13 +519,13 @@ __global__ void __launch_bounds__(1024) trow_plan_kernel(PlaceParams P) {
 template <int J>
 static size_t place_smem(int nj) {
   const size_t W = 32 * size_t(J ? J : nj), NW = kPlaceWarps;
-  return NW * (W * 12 + 32 * 48);
+  return NW * (W * (J ? 12 : 8) + 32 * 48);
 }
 
 template <int J, bool BWD>
 __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, int nj_dyn) {
   await_previous();
-  constexpr int NW = kPlaceWarps;
+  constexpr int NW = kPlaceWarps, U = 4;  // U: rows per lane and step of the run-time table's passes
   extern __shared__ __align__(16) unsigned char s_place[];
   __shared__ ViewTab T;
   const int nj = J ? J : nj_dyn, W = 32 * nj;
@@ -534,10 +534,11 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
   float4 *s_B = reinterpret_cast<float4 *>(s_place) + (NW + warp) * 32;               // det, hy, ydx, -
   uint4 *s_C = reinterpret_cast<uint4 *>(s_place) + (2 * NW + warp) * 32;             // start, ty0, tx0 | tx1 << 16, pos
   uint2 *mc = reinterpret_cast<uint2 *>(s_place + 48 * 32 * NW) + warp * W;           // masks and cursors
-  uint32_t *tog = reinterpret_cast<uint32_t *>(s_place + 48 * 32 * NW + 8 * NW * W) + warp * W;  // toggles
+  uint32_t *tog = reinterpret_cast<uint32_t *>(s_place + 48 * 32 * NW + 8 * NW * W) + warp * W;  // toggles (J > 0)
   const int tw_shift = 31 - __clz(P.tile_w);                        // tile widths are powers of two
   const float th = float(P.tile_h);
-  for (int i = lane; i < W; i += 32) tog[i] = 0u;
+  if (J)
+    for (int i = lane; i < W; i += 32) tog[i] = 0u;
   build_view_tab(P, T);
   const uint32_t nchunks = T.chunk0[P.n_views], cap = P.cap;
   uint32_t kept = 0;
@@ -558,20 +559,19 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
     load_ids(ck.q0 + 32 + lane, info1, pos1, id1);
     if (ck.q0 + lane < b) el = P.ell[id0];
     uint32_t cur[J ? J : 1];
-    {
-      const uint32_t *cnt1 = P.cnt1 + size_t(T.entry0[ck.v]) + ck.cc;
-      const uint2 *ranges = P.trow_ranges + cam.trow_base;
-      auto slot = [&](int x) {  // the bin's first list slot, at most cap
-        if (x >= R) return cap;
-        const uint32_t st = ranges[x].x, l = cnt1[size_t(x) * ck.nch];
-        return l < cap - st ? st + l : cap;
-      };
-      if (J) {
+    const uint32_t *cnt1 = P.cnt1 + size_t(T.entry0[ck.v]) + ck.cc;
+    const uint2 *ranges = P.trow_ranges + cam.trow_base;
+    auto slot = [&](int x) {  // the bin's first list slot, at most cap
+      if (x >= R) return cap;
+      const uint32_t st = ranges[x].x, l = cnt1[size_t(x) * ck.nch];
+      return l < cap - st ? st + l : cap;
+    };
+    if (J) {
 #pragma unroll
-        for (int j = 0; j < (J ? J : 1); ++j) cur[j] = slot(lane * nj + j);
-      } else {
-        for (int j = 0; j < nj; ++j) mc[lane * nj + j] = make_uint2(0u, slot(lane * nj + j));
-      }
+      for (int j = 0; j < (J ? J : 1); ++j) cur[j] = slot(lane * nj + j);
+    } else {
+      for (int i = lane; i < W; i += 32) mc[i] = make_uint2(0u, kCulled);  // no cursor yet
+      __syncwarp();
     }
     uint32_t e_run = 0;  // BWD: instances of this chunk so far
     for (uint32_t q = ck.q0; q < b; q += 32) {
@@ -580,8 +580,10 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
       const uint32_t inc = warp_incl_scan(rows), start = inc - rows;
       const uint32_t n_inst = __shfl_sync(0xffffffffu, inc, 31);
       if (valid) {
-        atomicXor(&tog[ty0], 1u << lane);
-        atomicXor(&tog[ty0 + rows], 1u << lane);
+        if (J) {
+          atomicXor(&tog[ty0], 1u << lane);
+          atomicXor(&tog[ty0 + rows], 1u << lane);
+        }
         const Band bd = band_of(el);
         s_A[lane] = make_float4(bd.cx, bd.cy, bd.a, bd.b);
         s_B[lane] = make_float4(bd.det, bd.hy, bd.ydx, 0.f);
@@ -592,7 +594,29 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
       info0 = info1; pos0 = pos1;
       load_ids(q + 64 + lane, info1, pos1, id1);
       __syncwarp();
-      bins_masks<J>(tog, mc, nj, cur);
+      if constexpr (J > 0) {
+        bins_masks<J>(tog, mc, cur);
+      } else {
+        // the first of the group's rows in a tile row also fetches its cursor, if the chunk had none there yet
+        uint32_t seen = 0;
+        for (uint32_t base = 0; base < n_inst; base += 32 * U) {
+          uint32_t ty[U], at[U];
+          bool fetch[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int k = instance_owner(start, valid, base + 32 * u, seen);
+            const uint32_t i = base + 32 * u + lane;
+            ty[u] = i < n_inst ? s_C[k].y + (i - s_C[k].x) : 0u;
+            fetch[u] = i < n_inst && atomicOr(&mc[ty[u]].x, 1u << k) == 0u && mc[ty[u]].y == kCulled;
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) at[u] = fetch[u] ? slot(int(ty[u])) : 0u;
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (fetch[u]) mc[ty[u]].y = at[u];
+        }
+        __syncwarp();
+      }
       uint32_t seen = 0;
       for (uint32_t base = 0; base < n_inst; base += 32) {
         int k = instance_owner(start, valid, base, seen);
@@ -653,6 +677,25 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
         }
       }
       __syncwarp();
+      if (!J) {  // the lowest row of each mask moves the cursor past them all
+        uint32_t seen = 0;
+        for (uint32_t base = 0; base < n_inst; base += 32 * U) {
+          uint32_t ty[U], n[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int k = instance_owner(start, valid, base + 32 * u, seen);
+            const uint32_t i = base + 32 * u + lane;
+            ty[u] = i < n_inst ? s_C[k].y + (i - s_C[k].x) : 0u;
+            const uint32_t m = i < n_inst ? mc[ty[u]].x : 0u;
+            n[u] = (m & ((1u << k) - 1u)) == 0u ? __popc(m) : 0u;
+          }
+          __syncwarp();
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (n[u]) mc[ty[u]] = make_uint2(0u, mc[ty[u]].y + n[u]);
+          __syncwarp();
+        }
+      }
     }
     if (BWD && lane == 0) P.e_base[c] = atomicAdd(&P.counters->n_partials, e_run);
   }
@@ -662,23 +705,36 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
 
 // ------------------------------------------------------------------------- launchers
 
-// Chunk lengths the plan allows: the counts (tile rows x chunks) stay within one word per
-// (primitive, view) pair, and `heads` + 1 per tile row.
-static uint32_t place_cp_lo(int max_rows) {
-  uint32_t cp = 64;
+// Pairs of the shortest chunk: the counts (tile rows x chunks) stay within one word per (primitive, view)
+// pair, and `heads` + 1 per tile row.  With more tile rows than the compiled tables hold, chunks of so many pairs
+// leave most of the chip idle: where the workspace may grow, they are as short as 64 MB of counts allow.
+uint32_t place_chunk_lo(uint64_t pairs, int max_rows, bool short_chunks) {
+  uint32_t cp = 64, lo = 64;
   while (cp < uint32_t(max_rows)) cp <<= 1;
-  return cp;
+  if (!short_chunks || bins_per_lane(max_rows) <= 9) return cp;
+  while (lo < cp && pairs / lo * uint64_t(max_rows) > std::max<uint64_t>(16 * pairs, uint64_t(16) << 20)) lo <<= 1;
+  return lo;
 }
 // Head chunks of a view, and one chunk that is not full.
 static uint64_t place_view_chunks(int n_views, uint64_t pairs, int heads) {
   const uint64_t n = n_views > 0 ? pairs / uint64_t(n_views) : 0;
-  return std::min<uint64_t>(uint64_t(heads), n / kHeadPairs + 1) + 1;
+  return std::min<uint64_t>(uint64_t(heads), n / place_head_pairs(heads) + 1) + 1;
 }
-uint64_t place_max_chunks(int n_views, uint64_t pairs, int max_rows, int heads) {
-  return pairs / place_cp_lo(max_rows) + uint64_t(n_views) * place_view_chunks(n_views, pairs, heads);
+// Head chunks of a plan, of 2,048 pairs of a view in all: on views with more tile rows than the compiled
+// tables hold its nearest pairs have up to thousands of rows each, and there are four times as many where the
+// workspace may grow (64 MB of counts).
+int place_heads(int max_rows, int64_t trows, bool short_chunks) {
+  int heads = kHeadChunks;
+  if (short_chunks && bins_per_lane(max_rows) > 9)
+    while (heads < 4 * kHeadChunks && trows * heads * 2 <= int64_t(16) << 20) heads *= 2;
+  return heads;
 }
-uint64_t place_max_counts(int n_views, uint64_t pairs, int max_rows, int64_t trows, int heads) {
-  return pairs / place_cp_lo(max_rows) * uint64_t(max_rows) + uint64_t(trows) * place_view_chunks(n_views, pairs, heads);
+uint32_t place_head_pairs(int heads) { return heads > kHeadChunks ? uint32_t(16 * kHeadChunks / heads) : 16u; }
+uint64_t place_max_chunks(int n_views, uint64_t pairs, uint32_t chunk_lo, int heads) {
+  return pairs / chunk_lo + uint64_t(n_views) * place_view_chunks(n_views, pairs, heads);
+}
+uint64_t place_max_counts(int n_views, uint64_t pairs, int max_rows, int64_t trows, uint32_t chunk_lo, int heads) {
+  return pairs / chunk_lo * uint64_t(max_rows) + uint64_t(trows) * place_view_chunks(n_views, pairs, heads);
 }
 
 template <int J, bool BWD>
@@ -701,11 +757,11 @@ static cudaError_t run_place(const PlaceParams &P, int nj, int num_sms, uint64_t
 
 cudaError_t launch_place(PlaceParams P, int num_sms, cudaStream_t st) {
   if (P.trows == 0) return cudaSuccess;
-  P.cp_lo = place_cp_lo(P.max_rows);
   P.cp_hi = std::max(256u, P.cp_lo);
+  P.head_pairs = place_head_pairs(int(P.heads));
   P.target = uint32_t(num_sms) * 32;
   const uint64_t max_chunks =
-      std::max<uint64_t>(1, place_max_chunks(P.n_views, uint64_t(P.n) * uint64_t(P.n_views), P.max_rows, int(P.heads)));
+      std::max<uint64_t>(1, place_max_chunks(P.n_views, uint64_t(P.n) * uint64_t(P.n_views), P.cp_lo, int(P.heads)));
   const int nj = bins_per_lane(P.max_rows);
   const bool bwd = P.row_e != nullptr;
 #define RAYGS_PLACE(J) \
