@@ -53,29 +53,34 @@ bool fit_scratch(Work &w) {
   opt.tile_stop = false;
   opt.bin_once = true;
   opt.short_chunks = w.short_chunks = false;
-  int64_t most = 0;  // what the barest layout leaves
-  for (int i : {2, 0, 1, 2}) {
+  auto layout = [&](int64_t cap) {
+    w.cap = cap;
+    w.L = make_layout(w.n_views, w.n, w.tiles, w.trows, cap, w.num_sms, w.max_tiles_x, w.max_rows, opt);
+    return w.L.total <= kNoAllocScratchBytes;
+  };
+  double room = 0.0;
+  // The capacity that the i-th choice leaves, but for the rounding of the buffers.
+  auto guess = [&](int i) {
     opt.tile_order = keep[i].order;
     opt.heads = w.heads = keep[i].heads;
     opt.list_lo = w.list_lo = keep[i].list_lo;
-    auto layout = [&](int64_t cap) {
-      w.cap = cap;
-      w.L = make_layout(w.n_views, w.n, w.tiles, w.trows, cap, w.num_sms, w.max_tiles_x, w.max_rows, opt);
-      return w.L.total <= kNoAllocScratchBytes;
-    };
     layout(0);
-    const double room = double(kNoAllocScratchBytes) - double(w.L.total);
+    room = double(kNoAllocScratchBytes) - double(w.L.total);
     // the column counts: up to so many bytes per unit of capacity, and no more than so many in all
     const double per_unit = 4.0 * w.max_tiles_x / w.list_lo, in_all = 4.0 * w.max_tiles_x * list_target(w.num_sms);
-    int64_t cap = int64_t(std::max(room / (kBytesPerCapacity + per_unit), (room - in_all) / kBytesPerCapacity));
-    if (most == 0) {
-      if (cap <= 0) return false;
-      most = cap;
-      continue;
-    }
+    return int64_t(std::max(room / (kBytesPerCapacity + per_unit), (room - in_all) / kBytesPerCapacity));
+  };
+  auto fits = [&](int64_t cap) {
     while (cap > 0 && !layout(cap)) cap -= 256;
-    if (cap > 0 && (3 * cap >= 2 * most || i == 2)) return true;
-  }
+    return cap > 0;
+  };
+  // the usual case: two thirds of all that is left besides what the choices differ in
+  int64_t cap = guess(0);
+  const double extras = 4.0 * kTileClasses * double(w.tiles) + double(w.L.rows - w.L.cnt1);
+  if (cap > 0 && 3.0 * kBytesPerCapacity * double(cap) >= 2.0 * (room + extras) && fits(cap)) return true;
+  const int64_t most = guess(2);
+  for (int i = 0; i < 3 && most > 0; ++i)
+    if (3 * (cap = guess(i)) >= 2 * most && fits(cap)) return true;
   return false;
 }
 
