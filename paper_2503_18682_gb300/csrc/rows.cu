@@ -707,12 +707,14 @@ __global__ void __launch_bounds__(32 * kPlaceWarps) place_kernel(PlaceParams P, 
 
 // Pairs of the shortest chunk: the counts (tile rows x chunks) stay within one word per (primitive, view)
 // pair, and `heads` + 1 per tile row.  With more tile rows than the compiled tables hold, chunks of so many pairs
-// leave most of the chip idle: where the workspace may grow, they are as short as 64 MB of counts allow.
+// leave most of the chip idle: where the workspace may grow, they are as short as 64 MB of counts allow, or
+// 16 words per pair up to 256 MB.
 uint32_t place_chunk_lo(uint64_t pairs, int max_rows, bool short_chunks) {
   uint32_t cp = 64, lo = 64;
   while (cp < uint32_t(max_rows)) cp <<= 1;
   if (!short_chunks || bins_per_lane(max_rows) <= 9) return cp;
-  while (lo < cp && pairs / lo * uint64_t(max_rows) > std::max<uint64_t>(16 * pairs, uint64_t(16) << 20)) lo <<= 1;
+  const uint64_t words = std::max({pairs, std::min<uint64_t>(16 * pairs, uint64_t(64) << 20), uint64_t(16) << 20});
+  while (lo < cp && pairs / lo * uint64_t(max_rows) > words) lo <<= 1;
   return lo;
 }
 // Head chunks of a view, and one chunk that is not full.
